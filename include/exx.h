@@ -99,9 +99,10 @@ typedef struct {
     int threads;       /* threads per CTA, 0 = library choice, else a multiple of
                           32 in [256, 1024]; the one-CTA solver runs 256, 512
                           or 1024 (other values: the library choice, 512, or
-                          256 for the FP32 multigrid CG, which then keeps six
-                          CTAs per SM, five with per-pair radii), the cluster
-                          solver only the launch shapes it is built for.      */
+                          for the FP32 multigrid CG 128, 256 or 512 by the
+                          size of the pair's ball, 256 or 512 for the largest
+                          of the context), the cluster solver only the launch
+                          shapes it is built for.                             */
     int ctas_per_sm;   /* resident CTAs per SM, 0 = library choice (the
                           multigrid CG on clusters: 1 or 2, default 2).         */
     int solver_kind;   /* 0 = library choice; 1 = one CTA per pair with state in
@@ -144,7 +145,8 @@ typedef struct {
     int r_pe_nonself;  /* radii_mode 2: R_PE of non-self pairs, 1..R_PE        */
     int r_me_nonself;  /* radii_mode 2: R_ME of non-self pairs,
                           r_pe_nonself + 3 .. R_ME                              */
-    int fixed_residual;/* cluster solver with lane map 4 or 5 on an isotropic
+    int fixed_residual;/* cluster solver with lane map 4 or 5, and the FP32
+                          multigrid CG on one CTA per pair, on an isotropic
                           grid: 0 = the FP64 residuals of the refinement come
                           from an exact integer stencil on a fixed-point copy
                           of v (default), 1 = from the FP64 stencil, 2 = test

@@ -37,6 +37,10 @@ cudaError_t set_multipole_const_cluster(const MultipoleConst& mc);
 size_t pair_kernel_smem(int Rc, int r_pe_max);
 cudaError_t launch_pair_kernel(const SolveParams& P, int threads, bool mixed, int grid, size_t smem, cudaStream_t st);
 cudaError_t pair_kernel_occupancy(int threads, bool mixed, bool mg, bool one_ball, size_t smem, int* blocks_per_sm);
+cudaError_t set_multipole_const_march(const MultipoleConst& mc);
+cudaError_t march_occupancy(int threads, size_t smem, int* blocks_per_sm);
+cudaError_t launch_march_kernel(const SolveParams& P, int threads, int grid, size_t smem, cudaStream_t st);
+cudaError_t launch_class_runs(const int* hist, int n_geo, const int2* range, int n_class, int* cls, cudaStream_t st);
 cudaError_t launch_mg_apply(const SolveParams& P, int geo, const double* r, double* z, cudaStream_t st);  // exx_debug.cu
 cudaError_t launch_debug_readback(const SolveParams& P, const PairRec& pr, double* rho_me, double* v_me,
                                   cudaStream_t st);
@@ -126,6 +130,22 @@ struct exx_ctx {
     // the multigrid-preconditioned CG on clusters (preconditioner 1, precision 1):
     // mg_C CTAs per pair, mg_minb CTAs per SM, up to mg_clusters resident clusters
     int mg_C = 0, mg_minb = 2, mg_clusters = 0;
+    // the marching multigrid CG (exx_march.cu; preconditioner 1, precision 1,
+    // solver_kind 0 or 1): one launch per CTA size, the largest balls first,
+    // side by side on the context stream and the aux streams; each launch has
+    // its own workspace slots
+    struct MarchClass {
+        int threads = 0, g_lo = 0, g_hi = 0, slots = 0;
+        size_t smem = 0, at = 0, hot = 0;  // dynamic shared memory; first bytes of its slots
+        SolveParams P;            // slot offsets and sizes of the class (the rest as in the context's P)
+    };
+    std::vector<MarchClass> march;
+    char* march_ws = nullptr;
+    void* march_mem = nullptr;   // device tables
+    int2* d_march_range = nullptr;
+    int* d_march_cls = nullptr;  // [2 classes] start and length in the order, [classes] work counters
+    cudaStream_t march_st[5] = {};
+    cudaEvent_t march_ev[6] = {};  // joins of the aux streams, [5] fork
     // exx_compute_async: the last call's counters are read (after waiting for
     // the call) by the next exx_get_stats; box of that call
     bool stats_pending = false;
@@ -406,6 +426,13 @@ extern "C" void exx_destroy(exx_ctx* c) {
         if (e) cudaEventDestroy(e);
     for (auto& e : c->ev)
         if (e) cudaEventDestroy(e);
+    cudaFree(c->march_ws);
+    cudaFree(c->march_mem);
+    cudaFree(c->d_march_cls);
+    for (auto& e : c->march_ev)
+        if (e) cudaEventDestroy(e);
+    for (auto& q : c->march_st)
+        if (q) cudaStreamDestroy(q);
     if (c->ev_fork) cudaEventDestroy(c->ev_fork);
     if (c->ev_join) cudaEventDestroy(c->ev_join);
     if (c->aux) cudaStreamDestroy(c->aux);
@@ -413,6 +440,134 @@ extern "C" void exx_destroy(exx_ctx* c) {
     if (c->ev_out) cudaEventDestroy(c->ev_out);
     if (c->work) cudaStreamDestroy(c->work);
     delete c;
+}
+
+// CTA size of the marching multigrid CG for a ball of n columns: one each.
+static int march_threads(int n) { return n <= 128 ? 128 : (n <= 256 ? 256 : 512); }
+
+// Plans the marching multigrid CG: classes of radii by CTA size, tables and
+// slot layouts. Leaves c->march empty when a ball has no coarse level or is
+// larger than the largest CTA holds, or when the requested threads do not hold
+// the largest ball's columns (pair_kernel then runs the call).
+static exx_status plan_march(exx_ctx* c, const std::vector<std::vector<HostMGLevel>>& mgl) {
+    const int ng = c->n_geo, want = c->opt.threads;
+    const bool asked = want == 256 || want == 512 || want == 1024;
+    std::vector<HostMarch> H(ng);
+    std::vector<int> nt(ng);
+    const int largest = march_threads(march_columns(c->balls[ng - 1].r_pe));
+    for (int g = 0; g < ng; ++g) {
+        nt[g] = asked ? want : march_threads(march_columns(c->balls[g].r_pe));
+        if (!asked && nt[g] == largest) nt[g] = std::max(nt[g], 256);  // the largest ball's class
+        if (c->balls[g].r_pe > 35 || !build_march(c->balls[g], mgl[g], c->delta, nt[g], H[g])) return EXX_OK;
+    }
+    // tables
+    size_t bytes = align256(sizeof(MarchGeo) * ng) + align256(sizeof(int2) * ng);
+    for (const HostMarch& h : H) {
+        for (const HostMarchLv& l : h.lv) bytes += align256(sizeof(int) * l.col.size()) + align256(sizeof(int) * l.pst.size());
+        bytes += align256(sizeof(int) * h.qidx.size()) + align256(sizeof(int) * h.rim.size()) +
+                 align256(sizeof(int) * h.layer.size()) + align256(sizeof(double) * h.layer_ir.size());
+    }
+    CK(cudaMalloc(&c->march_mem, bytes), "cudaMalloc(marching tables)");
+    std::vector<char> host(bytes, 0);
+    size_t at = align256(sizeof(MarchGeo) * ng) + align256(sizeof(int2) * ng);
+    auto put = [&](const std::vector<int>& v) -> char* {
+        std::memcpy(host.data() + at, v.data(), sizeof(int) * v.size());
+        char* p = (char*)c->march_mem + at;
+        at += align256(sizeof(int) * v.size());
+        return p;
+    };
+    for (HostMarch& h : H) {
+        for (int l = 0; l < (int)h.lv.size(); ++l) {
+            h.G.lv[l].col = (const int4*)put(h.lv[l].col);
+            h.G.lv[l].pst = (const int*)put(h.lv[l].pst);
+        }
+        h.G.qidx = (const int*)put(h.qidx);
+        h.G.rim = (const int*)put(h.rim);
+        h.G.layer = (const int*)put(h.layer);
+        h.G.layer_ir = (const double*)((char*)c->march_mem + at);
+        std::memcpy(host.data() + at, h.layer_ir.data(), sizeof(double) * h.layer_ir.size());
+        at += align256(sizeof(double) * h.layer_ir.size());
+    }
+    // classes, the largest balls first
+    for (int g = ng - 1; g >= 0;) {
+        exx_ctx::MarchClass K;
+        K.threads = nt[g];
+        K.g_hi = g;
+        while (g >= 0 && nt[g] == K.threads) --g;
+        K.g_lo = g + 1;
+        std::memset(&K.P, 0, sizeof(K.P));
+        const HostBall& B = c->balls[K.g_hi];
+        const size_t S3 = (size_t)(2 * c->r_me + 1) * (2 * c->r_me + 1) * (2 * c->r_me + 1);
+        size_t off = 0;
+        auto take = [&](size_t n) {
+            const size_t here = off;
+            off = align256(off + n);
+            return here;
+        };
+        K.P.off_vcube = take(sizeof(double) * S3);
+        K.P.off_rho = take(sizeof(double) * B.n_pe);
+        K.P.off_vfix = take(sizeof(long long) * S3);
+        K.P.off_sy = take(sizeof(double) * kNMono * (size_t)(2 * B.r_me + 1));
+        K.P.off_ush = take((sizeof(double) + sizeof(float)) * kNU * B.rows_me.size());
+        K.P.off_rows = take(sizeof(double) * 8 * B.rows_pe.size());
+        K.P.slot_bytes = off;
+        off = 0;
+        const size_t vec = 2 * sizeof(float4) * (size_t)march_row(K.threads);
+        take(vec * kMarchVectors);
+        size_t floats = 0;
+        for (int q = K.g_lo; q <= K.g_hi; ++q) {
+            MarchGeo& M = H[q].G;
+            floats = std::max(floats, (size_t)M.smem_floats);
+            for (int l = 1; l < M.nm; ++l) {  // of its own for every ball: zero off the ball for good
+                M.lv[l].rhs_off = (int)(take(vec / 2 + sizeof(float4) * (size_t)M.lv[l].nq) / sizeof(float4));
+                M.lv[l].z_off = (int)(take(vec / 2 + sizeof(float4) * (size_t)M.lv[l].nq) / sizeof(float4));
+            }
+        }
+        K.P.hot_bytes = off;
+        K.smem = std::max(sizeof(float) * floats, sizeof(double) * (size_t)(2 * B.r_pe + 1) * 28);
+        c->march.push_back(K);
+    }
+    if (c->march.size() > 6) return fail(c, EXX_EINVAL, "exx_init: too many marching classes");
+    std::vector<MarchGeo> mg;
+    for (HostMarch& h : H) mg.push_back(h.G);
+    std::memcpy(host.data(), mg.data(), sizeof(MarchGeo) * ng);
+    std::vector<int2> range;
+    for (const auto& K : c->march) range.push_back(make_int2(K.g_lo, K.g_hi));
+    std::memcpy(host.data() + align256(sizeof(MarchGeo) * ng), range.data(), sizeof(int2) * range.size());
+    CK(cudaMemcpy(c->march_mem, host.data(), bytes, cudaMemcpyHostToDevice), "cudaMemcpy(marching tables)");
+    c->P.march = (const MarchGeo*)c->march_mem;
+    c->d_march_range = (int2*)((char*)c->march_mem + align256(sizeof(MarchGeo) * ng));
+    // slots: every CTA that can be resident, within a quarter of the free memory
+    size_t free_b = 0, total_b = 0, need = 0;
+    cudaMemGetInfo(&free_b, &total_b);
+    for (auto& K : c->march) {
+        int bps = 0;
+        CK(march_occupancy(K.threads, K.smem, &bps), "occupancy query (marching kernel)");
+        if (bps < 1) return fail(c, EXX_ECUDA, "marching kernel does not fit on an SM");
+        K.slots = c->num_sms * (c->opt.ctas_per_sm > 0 ? std::min(c->opt.ctas_per_sm, bps) : bps);
+        need += K.slots * (K.P.slot_bytes + K.P.hot_bytes);
+    }
+    if (need > free_b / 4) {
+        const double f = 0.25 * (double)free_b / (double)need;
+        for (auto& K : c->march) K.slots = std::max(1, (int)(K.slots * f));
+    }
+    at = 0;
+    for (auto& K : c->march) {
+        K.hot = at;
+        at += K.slots * K.P.hot_bytes;
+    }
+    for (auto& K : c->march) {
+        K.at = at;
+        at += K.slots * K.P.slot_bytes;
+    }
+    CK(cudaMalloc(&c->march_ws, at), "cudaMalloc(marching workspace)");
+    CK(cudaMemset(c->march_ws, 0, at), "cudaMemset(marching workspace)");
+    CK(cudaMalloc(&c->d_march_cls, sizeof(int) * 18), "cudaMalloc(marching classes)");
+    for (size_t k = 0; k + 1 < c->march.size(); ++k)
+        CK(cudaStreamCreateWithFlags(&c->march_st[k], cudaStreamNonBlocking), "stream creation (marching classes)");
+    for (auto& ev : c->march_ev)
+        CK(cudaEventCreateWithFlags(&ev, cudaEventDisableTiming), "event creation (marching classes)");
+    return EXX_OK;
 }
 
 extern "C" exx_status exx_init(exx_ctx** out, const double cell[3], const int grid[3], double r_pair, int r_pe,
@@ -521,6 +676,7 @@ extern "C" exx_status exx_init(exx_ctx** out, const double cell[3], const int gr
     }
     e = set_multipole_const_solve(mc);
     if (e == cudaSuccess) e = set_multipole_const_cluster(mc);
+    if (e == cudaSuccess) e = set_multipole_const_march(mc);
     if (e == cudaSuccess) e = exx::unet::set_multipole_const_unet(mc);
     if (e != cudaSuccess) return bail(cuda_fail(c, e, "cudaMemcpyToSymbol(multipoles)"));
 
@@ -717,6 +873,11 @@ extern "C" exx_status exx_init(exx_ctx** out, const double cell[3], const int gr
         if (e != cudaSuccess) return bail(cuda_fail(c, e, "cudaMemcpy(multigrid tables)"));
         P.mg = c->d_mg;
         P.mg_omega = 0.8;
+    }
+
+    if (mg_levels > 0 && o.precision == 1 && o.solver_kind != 2) {
+        const exx_status sm = plan_march(c, mgl);
+        if (sm != EXX_OK) return bail(sm);
     }
 
     // cluster solver candidates: every cluster size, thread count and lane map
@@ -971,6 +1132,10 @@ extern "C" exx_status exx_init(exx_ctx** out, const double cell[3], const int gr
     cudaMemGetInfo(&free_b, &total_b);
     long long fit = (long long)(0.25 * (double)free_b / (double)c->slot_bytes);
     c->n_slots = (int)std::max(1LL, std::min(want, fit));
+    if (!c->march.empty()) {  // pair_kernel's slots serve single-pair and operator queries only
+        c->n_slots = 1;
+        c->threads = c->march[0].threads;
+    }
     if (c->per_class && c->n_slots < want) {  // not enough memory for two lanes: one lane, shared slots
         c->lane_slots[0] = c->n_slots;
         c->lane_slots[1] = 0;
@@ -1081,6 +1246,10 @@ extern "C" exx_status exx_init(exx_ctx** out, const double cell[3], const int gr
     c->stats.grid_ctas = c->use_cluster ? c->n_clusters * c->CL.C
                                         : (c->mg_C ? std::min(c->mg_clusters, c->n_slots) * c->mg_C : c->n_slots);
     c->stats.lane_map = c->use_cluster ? c->cands[c->cand].lane_map : 0;
+    if (!c->march.empty()) {
+        c->stats.grid_ctas = 0;
+        for (const auto& K : c->march) c->stats.grid_ctas += K.slots;
+    }
     c->stats.n_candidates = (int)c->cands.size();
     c->stats.threads = c->threads;
     *out = c;
@@ -1138,6 +1307,9 @@ static exx_status enqueue(exx_ctx* c, const double* orbitals, const double* cent
         CK(launch_radii_sort(c->d_pairs, c->d_scalars, c->d_hist, c->n_geo, c->d_order, c->num_sms, st,
                              c->per_class ? c->d_class : nullptr),
            "largest-first order");
+    if (c->march.size() > 1)
+        CK(launch_class_runs(c->d_hist, c->n_geo, c->d_march_range, (int)c->march.size(), c->d_march_cls, st),
+           "marching classes");
     if (c->cur_box)
         CK(launch_box_clip(c->d_pairs, c->d_scalars, c->cur_box, c->cur_bdim, c->grid, c->d_scalars + 12, c->num_sms,
                            st),
@@ -1178,7 +1350,38 @@ static exx_status enqueue(exx_ctx* c, const double* orbitals, const double* cent
     else if (c->mg_C)
         CK(launch_cluster_mg(c->mg_C, c->mg_minb, P, std::min(c->mg_clusters, c->n_slots), st),
            "cluster multigrid kernel");
-    else
+    else if (!c->march.empty()) {
+        // one launch per CTA size, side by side: the classes' CTAs share the SMs
+        const int nk = (int)c->march.size();
+        if (nk > 1) CK(cudaEventRecord(c->march_ev[5], st), "cudaEventRecord(fork)");
+        for (int k = 0; k < nk; ++k) {
+            const exx_ctx::MarchClass& K = c->march[k];
+            cudaStream_t ks = k ? c->march_st[k - 1] : st;
+            if (k) CK(cudaStreamWaitEvent(ks, c->march_ev[5], 0), "cudaStreamWaitEvent(fork)");
+            SolveParams Pk = P;
+            Pk.ws = c->march_ws + K.at;
+            Pk.slot_bytes = K.P.slot_bytes;
+            Pk.ws_hot = c->march_ws + K.hot;
+            Pk.hot_bytes = K.P.hot_bytes;
+            Pk.off_vcube = K.P.off_vcube;
+            Pk.off_rho = K.P.off_rho;
+            Pk.off_vfix = K.P.off_vfix;
+            Pk.off_sy = K.P.off_sy;
+            Pk.off_ush = K.P.off_ush;
+            Pk.off_rows = K.P.off_rows;
+            if (nk > 1) {
+                Pk.item_base = c->d_march_cls + 2 * k;
+                Pk.n_pair = c->d_march_cls + 2 * k + 1;
+                Pk.queue = c->d_march_cls + 2 * nk + k;
+            }
+            CK(launch_march_kernel(Pk, K.threads, (int)std::min<long long>(K.slots, (long long)n * (n + 1) / 2), K.smem, ks),
+               "marching pair kernel");
+            if (k) {
+                CK(cudaEventRecord(c->march_ev[k - 1], ks), "cudaEventRecord(join)");
+                CK(cudaStreamWaitEvent(st, c->march_ev[k - 1], 0), "cudaStreamWaitEvent(join)");
+            }
+        }
+    } else
         CK(launch_pair_kernel(P, c->threads, c->opt.precision == 1, c->n_slots, c->smem, st), "pair kernel");
     if (P.dfix != 0.0)
         CK(launch_dfix_convert(d_xx, (long long)n * c->cur_ostride, 1.0 / P.dfix, c->num_sms, st), "D_xx to FP64");

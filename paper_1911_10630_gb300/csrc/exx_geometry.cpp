@@ -557,4 +557,209 @@ bool build_mg_levels(int r_pe, const double delta[3], std::vector<HostMGLevel>& 
     return true;
 }
 
+// One level's columns, buffer layout and plane starts.
+static void build_march_level(int R, MarchLv& L, HostMarchLv& H) {
+    const int zq = (R + 3) / 4, zmin = -4 * zq;  // quads [zmin, zmin + 4), ...
+    const int nzq = R / 4 + zq + 1;
+    std::memset(&L, 0, sizeof(L));
+    L.R = R;
+    // rows padded by one quad that serves the next row too, an odd number of
+    // quads (rows then start in different bank groups); rows y from -(R + 4) to
+    // R + 4 (a column's pair of rows may begin or end one row off the ball),
+    // 12 floats before and after for the quads that reach past a row's end
+    L.pitch = 4 * ((nzq + 1) | 1);
+    L.planef = 24 + (2 * R + 9) * L.pitch;
+    L.org = 12 + (R + 4) * L.pitch - zmin;
+    struct Col { int y, z0, xm[8], reach, bank; };
+    std::vector<Col> rest;  // by reach, the farthest first
+    for (int y = -2 * ((R + 1) / 2); y <= R; y += 2)
+        for (int z0 = zmin; z0 <= R; z0 += 4) {
+            Col c;
+            c.y = y;
+            c.z0 = z0;
+            c.reach = -1;
+            c.bank = ((L.org + y * L.pitch + z0) / 4) & 7;
+            for (int e = 0; e < 8; ++e) {
+                const long yy = y + (e >> 2), z = z0 + (e & 3);
+                c.xm[e] = isqrt_floor((long)R * R - yy * yy - z * z);  // -1: never in the ball
+                c.reach = std::max(c.reach, c.xm[e]);
+            }
+            if (c.reach >= 0) rest.push_back(c);
+        }
+    std::stable_sort(rest.begin(), rest.end(), [](const Col& a, const Col& b) { return a.reach > b.reach; });
+    // dealt from the first 32 left over: the next column takes a bank group that
+    // its run of 8 has not, the one with the most columns among the 32
+    H.col.clear();
+    std::vector<int> ncol(R + 1, 0);
+    unsigned used = 0;
+    int pos = 0;
+    while (!rest.empty()) {
+        if (pos % 8 == 0) used = 0;
+        const size_t w = std::min<size_t>(32, rest.size());
+        int count[8] = {0};
+        for (size_t k = 0; k < w; ++k) ++count[rest[k].bank];
+        size_t pick = 0;
+        int best = -1;
+        for (size_t k = 0; k < w; ++k)
+            if (!(used >> rest[k].bank & 1u) && count[rest[k].bank] > best) {
+                best = count[rest[k].bank];
+                pick = k;
+            }
+        const Col c = rest[pick];
+        rest.erase(rest.begin() + pick);
+        used |= 1u << c.bank;
+        unsigned xm[2] = {0, 0};
+        for (int e = 0; e < 8; ++e) xm[e >> 2] |= (unsigned)(c.xm[e] + 1) << (8 * (e & 3));
+        H.col.push_back((L.org + c.y * L.pitch + c.z0) | (c.y + 64) << 16 | (c.z0 + 64) << 24);
+        H.col.push_back((int)xm[0]);
+        H.col.push_back((int)xm[1]);
+        H.col.push_back(0);
+        ++pos;
+        for (int x = 0; x <= c.reach; ++x) ncol[x] = pos;  // plane |x| = x holds the columns up to its last
+    }
+    L.ncol = pos;
+    H.pst.assign(2 * R + 1, 0);
+    int q = 0;
+    for (int x = -R; x <= R; ++x) {
+        H.pst[x + R] = q;
+        q += ncol[x < 0 ? -x : x];
+    }
+    L.nq = q;
+}
+
+int march_columns(int R) {
+    MarchLv L;
+    HostMarchLv H;
+    build_march_level(R, L, H);
+    return L.ncol;
+}
+
+// With at most max_groups groups at level 0.
+static bool build_march_groups(const HostBall& B, const std::vector<HostMGLevel>& levels, int threads, int max_groups,
+                               HostMarch& H) {
+    MarchGeo& G = H.G;
+    std::memset(&G, 0, sizeof(G));
+    H.lv.clear();
+    if (levels.empty()) return false;
+    G.L = (int)levels.size();
+    G.nm = 1;  // the first level in shared memory
+    while (G.nm < G.L && levels[G.nm - 1].R > (G.nm == 1 ? kMarchSmem1 : kMarchSmem)) ++G.nm;
+    if (G.nm > kMarchMax || levels[G.nm - 1].R > kMarchSmem) return false;
+    H.lv.resize(G.nm + 1);
+    std::vector<int> groups(G.nm), n32(G.nm + 1);
+    for (int l = 0; l <= G.nm; ++l) {
+        MarchLv& L = G.lv[l];
+        build_march_level(l == 0 ? B.r_pe : levels[l - 1].R, L, H.lv[l]);
+        n32[l] = (L.ncol + 31) & ~31;
+        if (n32[l] > threads || L.nq > march_row(threads)) return false;
+        if (l == G.nm) break;
+        // as many groups as the threads hold, each slab three coarse planes at least
+        const int nX = 2 * ((L.R + 1) / 2) + 1;
+        L.groups = groups[l] = std::max(1, std::min(std::min(threads / n32[l], l == 0 ? max_groups : 8), nX / 3));
+    }
+    for (int l = 0; l < G.nm; ++l)  // the sums to restrict, or the next level's staged planes
+        G.lv[l].xfloats = std::max(std::max(G.lv[l].planef, 8 * n32[l]), l + 1 < G.nm ? 2 * G.lv[l + 1].planef : 0);
+    auto place_level = [&](int l, int at) {
+        MarchLv& L = G.lv[l];
+        L.sm = at;
+        at += groups[l] * 2 * L.planef;
+        L.sm_x = at;
+        at += groups[l] * L.xfloats;
+        L.stage = at;
+        return at + groups[l] * 4 * n32[l] * 4;
+    };
+    auto place_small = [&](int at) {
+        for (int l = G.nm; l <= G.L; ++l) {
+            MarchSmall& s = G.sl[l];
+            const int n = (int)levels[l - 1].off.size();
+            s.R = levels[l - 1].R;
+            s.pitch = 2 * s.R + 4;
+            s.plane = s.pitch * s.pitch;
+            s.org = 3 + 3 * s.pitch + 3 * s.plane + s.R * (1 + s.pitch + s.plane);
+            s.cube = at;
+            at += ((2 * s.R + 7) * s.plane + 4 * s.pitch + 3) & ~3;
+            s.rhs = at;
+            at += l < G.L ? (n + 3) & ~3 : 128 + std::max(threads, 128);
+        }
+        return at;
+    };
+    for (int l = G.nm; l <= G.L; ++l) {
+        const int n = (int)levels[l - 1].off.size();
+        if (n > (l < G.L ? kMarchPts * threads : 128)) return false;
+    }
+    int at = place_level(0, 0);
+    G.planes_floats = groups[0] * 2 * G.lv[0].planef;
+    if (G.nm > 1) {  // the coarse levels' space overlaps level 0's: fewer groups if it would not fit
+        // what an SM gives each of the CTAs that 128 registers a thread allow
+        const int budget = (233472 / std::max(1, 512 / threads) - 1024 - 3072) / 4 - 192;
+        int end = 0;
+        for (;;) {
+            end = 0;
+            int widest = 1;
+            for (int l = 1; l < G.nm; ++l) {
+                end = place_level(l, end);
+                if (groups[l] > groups[widest]) widest = l;
+            }
+            end = place_small(end);
+            if (end <= std::max(at, budget) || groups[widest] == 1) break;
+            G.lv[widest].groups = --groups[widest];
+        }
+        G.coarse_floats = end;
+        at = std::max(at, end);
+    } else {
+        at = place_small(at);
+    }
+    G.smem_zero = at;
+    G.sm_op = at;
+    at += 32;
+    for (int l = 0; l <= G.nm; ++l) {
+        G.lv[l].sm_pst = at;
+        at += 2 * G.lv[l].R + 1;
+    }
+    G.smem_floats = at;
+    // level-0 index of each PE point
+    const MarchLv& L = G.lv[0];
+    const int R = B.r_pe;
+    std::vector<int> rank((size_t)L.planef, -1);
+    for (int c = 0; c < L.ncol; ++c) rank[H.lv[0].col[4 * c] & 0xffff] = c;
+    H.qidx.assign(B.n_pe, 0);
+    for (int k = 0; k < B.n_pe; ++k) {
+        const int x = (B.off[k] & 255) - 128, y = ((B.off[k] >> 8) & 255) - 128, z = ((B.off[k] >> 16) & 255) - 128;
+        const int j = y & 1, z0 = z - (z & 3);
+        H.qidx[k] = 4 * (j * march_row(threads) + H.lv[0].pst[x + R] + rank[L.org + (y - j) * L.pitch + z0]) + (z - z0);
+    }
+    return true;
+}
+
+bool build_march(const HostBall& B, const std::vector<HostMGLevel>& levels, const double delta[3], int threads,
+                 HostMarch& H) {
+    for (int groups = 8; groups >= 1; --groups) {  // as many as fit the shared memory of an SM
+        if (!build_march_groups(B, levels, threads, groups, H)) return false;
+        if (H.G.smem_floats > 55 * 1024) continue;
+        // the rim, and the shell layer with its 1 / r
+        H.rim.clear();
+        const int in2 = B.r_pe > 3 ? (B.r_pe - 3) * (B.r_pe - 3) : -1;
+        for (int pass = 0; pass < 2; ++pass) {
+            for (int k = 0; k < B.n_pe; ++k) {
+                const int x = (B.off[k] & 255) - 128, y = ((B.off[k] >> 8) & 255) - 128, z = ((B.off[k] >> 16) & 255) - 128;
+                if ((x * x + y * y + z * z > in2) == (pass == 0)) H.rim.push_back(k);
+            }
+            if (pass == 0) H.G.n_rim = (int)H.rim.size();
+        }
+        H.layer.clear();
+        H.layer_ir.clear();
+        for (int row = 0; row < (int)B.rows_me.size(); ++row) {
+            const RowRec& R = B.rows_me[row];
+            for (int z = R.zpe + 1; z <= std::min<int>(R.zn, R.zme); ++z) {
+                const double x = R.ox * delta[0], y = R.oy * delta[1], zz = z * delta[2];
+                H.layer.push_back(row << 8 | z);
+                H.layer_ir.push_back(1.0 / std::sqrt(x * x + y * y + zz * zz));
+            }
+        }
+        H.G.n_layer = (int)H.layer.size();
+        return true;
+    }
+    return false;
+}
+
 }  // namespace exx

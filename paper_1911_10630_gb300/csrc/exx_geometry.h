@@ -82,4 +82,24 @@ struct HostMGLevel {
 };
 bool build_mg_levels(int r_pe, const double delta[3], std::vector<HostMGLevel>& levels, std::vector<double>& minv);
 
+// Tables of the marching multigrid CG (MarchGeo) for the PE ball B and its
+// coarse levels: per marching level (and the first shared-memory level, whose
+// columns the restriction writes) the columns sorted by reach in |x| but for
+// a window of 32, from which they are dealt so that 8 consecutive ones lie in 8
+// distinct bank groups; qidx the level-0 index of each PE point. Fills G except for the device pointers and slot offsets. Returns false
+// if the ball has no coarse level or more marching levels than kMarchMax.
+struct HostMarchLv {
+    std::vector<int> col;       // 4 ints per column
+    std::vector<int> pst;
+};
+struct HostMarch {
+    MarchGeo G;
+    std::vector<HostMarchLv> lv;
+    std::vector<int> qidx, rim, layer;
+    std::vector<double> layer_ir;
+};
+int march_columns(int R);  // columns of a ball of radius R
+bool build_march(const HostBall& B, const std::vector<HostMGLevel>& levels, const double delta[3], int threads,
+                 HostMarch& H);
+
 }  // namespace exx

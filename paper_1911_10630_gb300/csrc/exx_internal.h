@@ -77,6 +77,53 @@ struct MGGeo {
     const float* minv32;    // the same in FP32 (FP32 V-cycle)
 };
 
+// The marching multigrid CG (exx_march.cuh). A ball's rows are cut into
+// 16-byte quads along z; the columns (two rows of a quad) are sorted by their
+// reach in |x|, so plane x holds the first columns of the list and a vector is
+// stored as quads j nq + pst[x + R] + column, j the row.
+// Level 1 marches from radius 6 on, the levels below it from 9: smaller ones
+// live in shared memory as cubes.
+constexpr int kMarchSmem1 = 5, kMarchSmem = 8;
+constexpr int kMarchMax = 3;    // marching levels at most (R_PE <= 35: 35, 18, 9)
+// A vector in the hot slot: two rows of march_row quads, a constant of the CTA
+// size (the quads of the largest ball that its threads hold), so that the
+// vectors' places are constants of the kernel; level 0's vectors in this order.
+constexpr int march_row(int threads) { return threads <= 128 ? 2816 : threads <= 256 ? 8704 : 23552; }
+enum { kMarchR = 0, kMarchP = 2, kMarchZ = 4, kMarchD = 5, kMarchAp = 6, kMarchVectors = 7 };  // R, P: two each
+constexpr int kMarchPts = 9;    // points per thread of a shared-memory level at most
+struct MarchLv {
+    int R, ncol, nq;            // radius, columns of plane 0, quads of one row of all columns
+    int pitch, planef, org;     // plane buffer: floats per row and in all, index of (y, z) = (0, 0)
+    int sm, sm_x, stage;        // first floats in shared memory: plane buffers ([groups][2]), the extra
+                                // buffer ([groups][xfloats]), staged inputs ([groups][4][threads] quads)
+    int xfloats;
+    int sm_pst;                 // first word of the plane starts there
+    int groups;                 // groups of threads that march the level, each a slab of planes
+    const int4* col;            // [ncol] buffer index | (y + 64) << 16 | (z0 + 64) << 24; per row bytes: |x| reach + 1
+    const int* pst;             // [2 R + 1] first quad of plane x
+    int rhs_off, z_off;         // levels >= 1, in the hot slot: first quads of right-hand side and correction
+};
+struct MarchSmall {             // a level in shared memory: zero-padded cube, compact right-hand side
+    int R, cube, rhs;           // radius, first floats
+    int org, plane, pitch;      // cube index of (X, Y, Z): org + X plane + Y pitch + Z
+};
+struct MarchGeo {
+    int nm, L;                  // marching levels 0 .. nm - 1; shared-memory levels nm .. L (L: dense inverse)
+    int smem_zero, smem_floats; // shared memory: floats zeroed per pair, in all
+    int sm_op;                  // the operator and the rings' address
+    int planes_floats;          // level 0's plane buffers, at 0
+    int coarse_floats;          // the coarse levels' space, at 0 too (nm > 1)
+    MarchLv lv[kMarchMax + 1];  // lv[nm]: only the columns of the first shared-memory level
+    MarchSmall sl[kMGMax + 1];
+    const int* qidx;            // [n_pe] index of each PE point in a level-0 vector
+    const int* rim;             // [n_pe] the PE points whose stencils reach the shell (n_rim), then the others
+    int n_rim;
+    // shell points that the stencil reads, z and -z as one: ME row << 8 | |z|, and 1 / r
+    const int* layer;
+    const double* layer_ir;
+    int n_layer;
+};
+
 // Everything the pair kernel needs, passed by value.
 struct SolveParams {
     // inputs / outputs
@@ -117,7 +164,7 @@ struct SolveParams {
     size_t off_sy;                                               // [C][(2 r_pe + 1) * 28] plane sums (cluster)
     size_t off_ush;                                              // [28][n_rows_me] FP64 then FP32 row coefficients U_{l,c} (cluster)
     size_t off_vfix;                                             // [S^3] int64 fixed-point copy of v (cluster, fixres)
-    int fixres;               // cluster kernel: FP64 residuals from an exact integer stencil on a fixed-point v
+    int fixres;               // cluster and marching kernels: FP64 residuals from an exact integer stencil on a fixed-point v
                               // (1; 2: bound made too small, every pair falls back, for tests)
     double fix_inv;           // 1 / (180 delta^2): the integer stencil's weights are 180 delta^2 x Eq. d2_1's
     double dfix;              // D_xx as fixed-point integers with this scale (2^40; 0 = FP64 atomics)
@@ -134,6 +181,11 @@ struct SolveParams {
     float mg_wd32[kMGMax + 1];
     size_t off_zc, off_tc;    // level-0 cubes (the workspace cube's size): smoothed correction, residual
     size_t off_mgz[kMGMax + 1], off_mgt[kMGMax + 1], off_mgr[kMGMax + 1];  // levels 1..: cubes and right-hand side
+    // marching multigrid CG: per geometry; the vectors its iterations stream,
+    // in slots of their own (the pairs in flight then span few pages)
+    const MarchGeo* march;
+    char* ws_hot;
+    size_t hot_bytes;
     const double* pow_tab;  // [3][2 Rc + 1][8] x^e, y^e, z^e (cluster kernel; global, read-only)
 
     // solver

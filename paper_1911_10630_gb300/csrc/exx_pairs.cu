@@ -229,6 +229,19 @@ __global__ void radii_classes_kernel(const int* __restrict__ hist, int n_geo, in
     }
 }
 
+// The same for ranges of geometries (class k takes range[k].x .. range[k].y):
+// the runs are adjacent in the order, the largest geometry first.
+__global__ void class_runs_kernel(const int* __restrict__ hist, int n_geo, const int2* __restrict__ range, int n_class,
+                                  int* __restrict__ cls) {
+    const int k = threadIdx.x;
+    if (k >= n_class) return;
+    const int2 r = range[k];
+    const int start = hist[n_geo + r.y] - hist[r.y];
+    cls[2 * k] = start;
+    cls[2 * k + 1] = hist[n_geo + r.x] - start;
+    cls[2 * n_class + k] = 0;
+}
+
 // Compact boxes: counts the pairs whose ME ball (the bounding cube of side
 // 2 R_ME + 1 around g_ij) is not inside both orbitals' boxes; for those the
 // result differs from the full-grid one (the orbitals count as zero outside).
@@ -364,6 +377,11 @@ cudaError_t launch_radii_sort(const PairRec* pairs, const int* n_pair, int* hist
     radii_scan_kernel<<<1, 32, 0, st>>>(hist, n_geo);
     radii_scatter_kernel<<<num_sms * 2, 256, 0, st>>>(pairs, n_pair, hist, n_geo, order);
     if (classes) radii_classes_kernel<<<1, 64, 0, st>>>(hist, n_geo, classes);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_class_runs(const int* hist, int n_geo, const int2* range, int n_class, int* cls, cudaStream_t st) {
+    class_runs_kernel<<<1, 32, 0, st>>>(hist, n_geo, range, n_class, cls);
     return cudaGetLastError();
 }
 
