@@ -106,7 +106,7 @@ typedef struct {
     int ctas_per_sm;   /* resident CTAs per SM, 0 = library choice (the
                           multigrid CG on clusters: 1 or 2, default 2).         */
     int solver_kind;   /* 0 = library choice; 1 = one CTA per pair with state in
-                          global memory; 2 = one thread-block cluster per pair
+                          global memory (the plain FP64 CG: 1 to 8); 2 = one thread-block cluster per pair
                           (plain CG: the FP32 inner state in shared memory;
                           multigrid CG: all state in the pair's workspace,
                           shared by the cluster's CTAs; only when requested). */
@@ -145,8 +145,10 @@ typedef struct {
     int r_pe_nonself;  /* radii_mode 2: R_PE of non-self pairs, 1..R_PE        */
     int r_me_nonself;  /* radii_mode 2: R_ME of non-self pairs,
                           r_pe_nonself + 3 .. R_ME                              */
-    int fixed_residual;/* cluster solver with lane map 4 or 5, and the FP32
-                          multigrid CG on one CTA per pair, on an isotropic
+    int fixed_residual;/* cluster solver with lane map 4 or 5, the FP32 multigrid
+                          CG on one CTA per pair, and A p of the plain FP64 CG
+                          (0 and 2 alike: 60 bits of p, rescaled each
+                          iteration, do not overflow), on an isotropic
                           grid: 0 = the FP64 residuals of the refinement come
                           from an exact integer stencil on a fixed-point copy
                           of v (default), 1 = from the FP64 stencil, 2 = test

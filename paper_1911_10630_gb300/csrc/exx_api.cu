@@ -38,6 +38,10 @@ size_t pair_kernel_smem(int Rc, int r_pe_max);
 cudaError_t launch_pair_kernel(const SolveParams& P, int threads, bool mixed, int grid, size_t smem, cudaStream_t st);
 cudaError_t pair_kernel_occupancy(int threads, bool mixed, bool mg, bool one_ball, size_t smem, int* blocks_per_sm);
 cudaError_t set_multipole_const_march(const MultipoleConst& mc);
+cudaError_t set_multipole_const_cg64(const MultipoleConst& mc);
+size_t cg64_smem(int r_pe);
+cudaError_t cg64_occupancy(int threads, bool fix, size_t smem, int* blocks_per_sm);
+cudaError_t launch_cg64_kernel(const SolveParams& P, int threads, bool fix, int teams, int team, size_t smem, cudaStream_t st);
 cudaError_t march_occupancy(int threads, size_t smem, int* blocks_per_sm);
 cudaError_t launch_march_kernel(const SolveParams& P, int threads, int grid, size_t smem, cudaStream_t st);
 cudaError_t launch_class_runs(const int* hist, int n_geo, const int2* range, int n_class, int* cls, cudaStream_t st);
@@ -130,6 +134,8 @@ struct exx_ctx {
     // the multigrid-preconditioned CG on clusters (preconditioner 1, precision 1):
     // mg_C CTAs per pair, mg_minb CTAs per SM, up to mg_clusters resident clusters
     int mg_C = 0, mg_minb = 2, mg_clusters = 0;
+    // the plain FP64 CG (exx_cg64.cu): CTAs that can be resident, 0 = not used
+    int cg64_ctas = 0;
     // the marching multigrid CG (exx_march.cu; preconditioner 1, precision 1,
     // solver_kind 0 or 1): one launch per CTA size, the largest balls first,
     // side by side on the context stream and the aux streams; each launch has
@@ -442,6 +448,38 @@ extern "C" void exx_destroy(exx_ctx* c) {
     delete c;
 }
 
+// 180 delta^2 times the stencil's weights are integers: the spacings are one, to
+// rounding (an operator of 1e-15 more or less).
+static bool isotropic(const exx_ctx* c) {
+    const double lo = std::min(c->delta[0], std::min(c->delta[1], c->delta[2]));
+    const double hi = std::max(c->delta[0], std::max(c->delta[1], c->delta[2]));
+    return hi - lo <= 4e-16 * hi;
+}
+static bool cg64_fixed(const exx_ctx* c) { return isotropic(c) && c->opt.fixed_residual != 1; }
+
+// CTAs per pair of the plain FP64 CG. Few pairs (at most n (n + 1) / 2) fill the
+// SMs by sharing: up to one CTA per SM in all, each thread with a pair of points
+// and a half at least, for the team's barriers (R_PE 16, 10 pairs: 7.1 / 4.5 /
+// 3.3 / 2.7 ms on teams of 1 / 2 / 4 / 8; 36: 7.5 / 4.8 / 3.5 / 4.3; R_PE 12, 21:
+// 3.3 / 2.4 / 2.0 / 2.5). With many pairs the barriers only pay on large balls,
+// whose pairs in flight then lie in L2 (R_PE 24, 177: 50 / 46 / 46 / 47; R_PE 20:
+// 27 / 28 / 25 / 27; R_PE 16, 210: 14 / 16 / 16 / 25; R_PE 8, 820: 5.4 / 8.6 / 16 / 32).
+static int cg64_team(const exx_ctx* c, int n) {
+    const long long pairs = (long long)n * (n + 1) / 2;
+    const size_t duos = c->hb.duo.size();
+    int team = 1;
+    while (team < 8 && pairs * 2 * team <= c->num_sms && duos >= (size_t)2 * team * 768) team *= 2;
+    return team == 1 && duos >= 20000 ? 2 : team;
+}
+static cudaError_t launch_cg64(exx_ctx* c, const SolveParams& P, int n, cudaStream_t st) {
+    const int team = cg64_team(c, n);
+    const int resident = std::max(1, c->cg64_ctas / team);
+    const int teams = (int)std::min<long long>(std::min(c->n_slots, resident), (long long)n * (n + 1) / 2);
+    c->stats.cluster_size = team;
+    c->stats.grid_ctas = teams * team;
+    return launch_cg64_kernel(P, c->threads, cg64_fixed(c), teams, team, c->smem, st);
+}
+
 // CTA size of the marching multigrid CG for a ball of n columns: one each.
 static int march_threads(int n) { return n <= 128 ? 128 : (n <= 256 ? 256 : 512); }
 
@@ -458,14 +496,13 @@ static exx_status plan_march(exx_ctx* c, const std::vector<std::vector<HostMGLev
     for (int g = 0; g < ng; ++g) {
         nt[g] = asked ? want : march_threads(march_columns(c->balls[g].r_pe));
         if (!asked && nt[g] == largest) nt[g] = std::max(nt[g], 256);  // the largest ball's class
-        if (c->balls[g].r_pe > 35 || !build_march(c->balls[g], mgl[g], c->delta, nt[g], H[g])) return EXX_OK;
+        if (c->balls[g].r_pe > 35 || !build_march(c->balls[g], mgl[g], nt[g], H[g])) return EXX_OK;
     }
     // tables
     size_t bytes = align256(sizeof(MarchGeo) * ng) + align256(sizeof(int2) * ng);
     for (const HostMarch& h : H) {
         for (const HostMarchLv& l : h.lv) bytes += align256(sizeof(int) * l.col.size()) + align256(sizeof(int) * l.pst.size());
-        bytes += align256(sizeof(int) * h.qidx.size()) + align256(sizeof(int) * h.rim.size()) +
-                 align256(sizeof(int) * h.layer.size()) + align256(sizeof(double) * h.layer_ir.size());
+        bytes += align256(sizeof(int) * h.qidx.size());
     }
     CK(cudaMalloc(&c->march_mem, bytes), "cudaMalloc(marching tables)");
     std::vector<char> host(bytes, 0);
@@ -482,11 +519,6 @@ static exx_status plan_march(exx_ctx* c, const std::vector<std::vector<HostMGLev
             h.G.lv[l].pst = (const int*)put(h.lv[l].pst);
         }
         h.G.qidx = (const int*)put(h.qidx);
-        h.G.rim = (const int*)put(h.rim);
-        h.G.layer = (const int*)put(h.layer);
-        h.G.layer_ir = (const double*)((char*)c->march_mem + at);
-        std::memcpy(host.data() + at, h.layer_ir.data(), sizeof(double) * h.layer_ir.size());
-        at += align256(sizeof(double) * h.layer_ir.size());
     }
     // classes, the largest balls first
     for (int g = ng - 1; g >= 0;) {
@@ -677,6 +709,7 @@ extern "C" exx_status exx_init(exx_ctx** out, const double cell[3], const int gr
     e = set_multipole_const_solve(mc);
     if (e == cudaSuccess) e = set_multipole_const_cluster(mc);
     if (e == cudaSuccess) e = set_multipole_const_march(mc);
+    if (e == cudaSuccess) e = set_multipole_const_cg64(mc);
     if (e == cudaSuccess) e = exx::unet::set_multipole_const_unet(mc);
     if (e != cudaSuccess) return bail(cuda_fail(c, e, "cudaMemcpyToSymbol(multipoles)"));
 
@@ -705,12 +738,14 @@ extern "C" exx_status exx_init(exx_ctx** out, const double cell[3], const int gr
             Rm = g == 0 ? o.r_me_nonself : r_me;
         }
         build_ball(c->balls[g], R, Rm, Rc);
+        build_ball_layers(c->balls[g], Rc, c->delta);
     }
     c->hb = c->balls.back();
     const HostBall& B = c->hb;
     {
         std::vector<size_t> o_cube(c->n_geo), o_off(c->n_geo), o_rpe(c->n_geo), o_rme(c->n_geo), o_pl(c->n_geo),
-            o_ro(c->n_geo), o_sn(c->n_geo), o_sf(c->n_geo);
+            o_ro(c->n_geo), o_sn(c->n_geo), o_sf(c->n_geo), o_rim(c->n_geo), o_lay(c->n_geo), o_ir(c->n_geo),
+            o_bd(c->n_geo), o_bc(c->n_geo);
         size_t at = 0;
         for (int g = 0; g < c->n_geo; ++g) {
             const HostBall& Bg = c->balls[g];
@@ -722,6 +757,11 @@ extern "C" exx_status exx_init(exx_ctx** out, const double cell[3], const int gr
             o_ro[g] = at; at = align256(at + sizeof(int) * Bg.row_of.size());
             o_sn[g] = at; at = align256(at + sizeof(int) * Bg.sh_near.size());
             o_sf[g] = at; at = align256(at + sizeof(int) * Bg.sh_far.size());
+            o_rim[g] = at; at = align256(at + sizeof(int) * Bg.rim.size());
+            o_lay[g] = at; at = align256(at + sizeof(int) * Bg.layer.size());
+            o_ir[g] = at; at = align256(at + sizeof(double) * Bg.layer_ir.size());
+            o_bd[g] = at; at = align256(at + sizeof(int) * Bg.duo.size());
+            o_bc[g] = at; at = align256(at + sizeof(int) * Bg.duo_k.size());
         }
         const size_t o_geo = at;
         const size_t geo_bytes = align256(o_geo + sizeof(BallGeo) * c->n_geo);
@@ -748,6 +788,14 @@ extern "C" exx_status exx_init(exx_ctx** out, const double cell[3], const int gr
             G.sh_far = (const int*)(gm + o_sf[g]);
             G.n_near = (int)Bg.sh_near.size();
             G.n_far = (int)Bg.sh_far.size();
+            G.rim = (const int*)(gm + o_rim[g]);
+            G.n_rim = Bg.n_rim;
+            G.layer = (const int*)(gm + o_lay[g]);
+            G.layer_ir = (const double*)(gm + o_ir[g]);
+            G.n_layer = (int)Bg.layer.size();
+            G.duo = (const int*)(gm + o_bd[g]);
+            G.duo_k = (const int2*)(gm + o_bc[g]);
+            G.n_duo = (int)Bg.duo.size();
             if ((e = cudaMemcpy(gm + o_ro[g], Bg.row_of.data(), sizeof(int) * Bg.row_of.size(), cudaMemcpyHostToDevice)) != cudaSuccess ||
                 (e = cudaMemcpy(gm + o_cube[g], Bg.cube.data(), sizeof(int) * Bg.n_me, cudaMemcpyHostToDevice)) != cudaSuccess ||
                 (e = cudaMemcpy(gm + o_off[g], Bg.off.data(), sizeof(int) * Bg.n_me, cudaMemcpyHostToDevice)) != cudaSuccess ||
@@ -755,7 +803,12 @@ extern "C" exx_status exx_init(exx_ctx** out, const double cell[3], const int gr
                 (e = cudaMemcpy(gm + o_rme[g], Bg.rows_me.data(), sizeof(RowRec) * Bg.rows_me.size(), cudaMemcpyHostToDevice)) != cudaSuccess ||
                 (e = cudaMemcpy(gm + o_pl[g], Bg.plane_pe.data(), sizeof(int) * Bg.plane_pe.size(), cudaMemcpyHostToDevice)) != cudaSuccess ||
                 (e = cudaMemcpy(gm + o_sn[g], Bg.sh_near.data(), sizeof(int) * Bg.sh_near.size(), cudaMemcpyHostToDevice)) != cudaSuccess ||
-                (e = cudaMemcpy(gm + o_sf[g], Bg.sh_far.data(), sizeof(int) * Bg.sh_far.size(), cudaMemcpyHostToDevice)) != cudaSuccess)
+                (e = cudaMemcpy(gm + o_sf[g], Bg.sh_far.data(), sizeof(int) * Bg.sh_far.size(), cudaMemcpyHostToDevice)) != cudaSuccess ||
+                (e = cudaMemcpy(gm + o_rim[g], Bg.rim.data(), sizeof(int) * Bg.rim.size(), cudaMemcpyHostToDevice)) != cudaSuccess ||
+                (e = cudaMemcpy(gm + o_bd[g], Bg.duo.data(), sizeof(int) * Bg.duo.size(), cudaMemcpyHostToDevice)) != cudaSuccess ||
+                (e = cudaMemcpy(gm + o_bc[g], Bg.duo_k.data(), sizeof(int) * Bg.duo_k.size(), cudaMemcpyHostToDevice)) != cudaSuccess ||
+                (e = cudaMemcpy(gm + o_lay[g], Bg.layer.data(), sizeof(int) * Bg.layer.size(), cudaMemcpyHostToDevice)) != cudaSuccess ||
+                (e = cudaMemcpy(gm + o_ir[g], Bg.layer_ir.data(), sizeof(double) * Bg.layer_ir.size(), cudaMemcpyHostToDevice)) != cudaSuccess)
                 return bail(cuda_fail(c, e, "cudaMemcpy(geometry)"));
         }
         c->geo_host = gv.back();
@@ -783,17 +836,18 @@ extern "C" exx_status exx_init(exx_ctx** out, const double cell[3], const int gr
     std::memset(&P, 0, sizeof(P));
     size_t off = 0;
     P.off_vcube = off; off = align256(off + sizeof(double) * S3);
-    P.off_pcube = off; off = align256(off + sizeof(double) * S3);
+    P.off_pcube = off; off = align256(off + sizeof(double) * (S3 + (long long)S * S));
     P.off_p32 = off; off = align256(off + sizeof(float) * S3);
     P.off_rho = off; off = align256(off + sizeof(double) * B.n_pe);
-    P.off_r = off; off = align256(off + sizeof(double) * B.n_pe);
-    P.off_d = off; off = align256(off + sizeof(double) * B.n_pe);
-    P.off_ap = off; off = align256(off + sizeof(double) * B.n_pe);
+    const size_t nv = std::max<size_t>(B.n_pe, 2 * B.duo.size());
+    P.off_r = off; off = align256(off + sizeof(double) * nv);
+    P.off_d = off; off = align256(off + sizeof(double) * nv);
+    P.off_ap = off; off = align256(off + sizeof(double) * nv);
     P.off_r32 = off; off = align256(off + sizeof(float) * B.n_pe);
     P.off_d32 = off; off = align256(off + sizeof(float) * B.n_pe);
     P.off_ap32 = off; off = align256(off + sizeof(float) * B.n_pe);
     P.off_rows = off; off = align256(off + sizeof(double) * 8 * B.rows_pe.size());
-    P.off_sy = off; off = align256(off + sizeof(double) * (size_t)kMaxCluster * (((2 * r_pe + 1) * 28 + 1) & ~1));
+    P.off_sy = off; off = align256(off + sizeof(double) * std::max((size_t)kMaxCluster * (((2 * r_pe + 1) * 28 + 1) & ~1), (size_t)kNMono * (2 * r_me + 1)));
     P.off_ush = off; off = align256(off + (sizeof(double) + sizeof(float)) * kNU * B.rows_me.size());
     P.off_vfix = off; off = align256(off + sizeof(long long) * S3);
     if (mg_levels > 0) {
@@ -1118,6 +1172,13 @@ extern "C" exx_status exx_init(exx_ctx** out, const double cell[3], const int gr
             c->lane_slots[lane] = std::max(c->lane_slots[lane], need);
         }
         want = (long long)c->lane_slots[0] + c->lane_slots[1];
+    } else if (o.precision == 0 && !P.mg) {
+        c->smem = cg64_smem(r_pe);
+        e = cg64_occupancy(c->threads, cg64_fixed(c), c->smem, &bps);
+        if (e != cudaSuccess) return bail(cuda_fail(c, e, "occupancy query"));
+        if (bps < 1) return bail(fail(c, EXX_ECUDA, "pair kernel does not fit on an SM"));
+        c->cg64_ctas = c->num_sms * (o.ctas_per_sm > 0 ? std::min(o.ctas_per_sm, bps) : bps);
+        want = c->cg64_ctas;
     } else {
         e = pair_kernel_occupancy(c->threads, o.precision == 1, o.preconditioner == 1, c->n_geo == 1, c->smem, &bps);
         if (e != cudaSuccess) return bail(cuda_fail(c, e, "occupancy query"));
@@ -1183,10 +1244,10 @@ extern "C" exx_status exx_init(exx_ctx** out, const double cell[3], const int gr
     double inv2[3];
     for (int a = 0; a < 3; ++a) inv2[a] = 1.0 / (c->delta[a] * c->delta[a]);
     // isotropic grids: 180 delta^2 x the weights are the integers -490, 270, -27, 2
-    P.fixres = (c->delta[0] == c->delta[1] && c->delta[1] == c->delta[2] && c->opt.fixed_residual != 1)
+    P.fixres = (isotropic(c) && c->opt.fixed_residual != 1)
                    ? (c->opt.fixed_residual == 2 ? 2 : 1)
                    : 0;
-    P.fix_inv = inv2[0] / 180.0;
+    P.fix_inv = (inv2[0] + inv2[1] + inv2[2]) / 540.0;
     P.dfix = c->opt.deterministic ? 1099511627776.0 : 0.0;  // 2^40
     P.st64.c0 = W[0] * (inv2[0] + inv2[1] + inv2[2]);
     for (int q = 1; q <= 3; ++q) {
@@ -1382,7 +1443,9 @@ static exx_status enqueue(exx_ctx* c, const double* orbitals, const double* cent
             }
         }
     } else
-        CK(launch_pair_kernel(P, c->threads, c->opt.precision == 1, c->n_slots, c->smem, st), "pair kernel");
+        CK(c->cg64_ctas ? launch_cg64(c, P, n, st)
+                        : launch_pair_kernel(P, c->threads, c->opt.precision == 1, c->n_slots, c->smem, st),
+           "pair kernel");
     if (P.dfix != 0.0)
         CK(launch_dfix_convert(d_xx, (long long)n * c->cur_ostride, 1.0 / P.dfix, c->num_sms, st), "D_xx to FP64");
     CK(cudaEventRecordWithFlags(c->ev[2], st, evf), "cudaEventRecord");
@@ -2037,6 +2100,7 @@ extern "C" exx_status exx_debug_pair(exx_ctx* c, const double* orbitals, int ind
     P.dbg_b = d_b;
     exx_status s = EXX_OK;
     cudaError_t e = c->use_cluster ? launch_cluster_kernel(c->cl_variant, P, c->CL, 1, c->smem, st)
+                    : c->cg64_ctas ? launch_cg64(c, P, 1, st)
                                    : launch_pair_kernel(P, c->threads, c->opt.precision == 1, 1, c->smem, st);
     if (e == cudaSuccess) e = launch_debug_readback(P, pr, d_rho, d_v, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);

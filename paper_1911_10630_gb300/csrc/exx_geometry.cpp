@@ -178,6 +178,43 @@ void build_ball(HostBall& B, int r_pe, int r_me, int Rc) {
     B.n_me = (int)B.cube.size();
 }
 
+// The PE ball's rim first, and the shell layer that its stencils read with 1 / r.
+void build_ball_layers(HostBall& B, int Rc, const double delta[3]) {
+    B.rim.clear();
+    const int in2 = B.r_pe > 3 ? (B.r_pe - 3) * (B.r_pe - 3) : -1;
+    for (int pass = 0; pass < 2; ++pass) {
+        for (int k = 0; k < B.n_pe; ++k) {
+            const int x = (B.off[k] & 255) - 128, y = ((B.off[k] >> 8) & 255) - 128, z = ((B.off[k] >> 16) & 255) - 128;
+            if ((x * x + y * y + z * z > in2) == (pass == 0)) B.rim.push_back(k);
+        }
+        if (pass == 0) B.n_rim = (int)B.rim.size();
+    }
+    B.duo.clear();
+    B.duo_k.clear();
+    const int S = 2 * Rc + 1;
+    for (int lo = -B.r_pe; lo <= B.r_pe; lo += kBand)
+        for (const RowRec& R : B.rows_pe) {
+            if (R.oy < lo || R.oy >= lo + kBand) continue;
+            const int c0 = ((R.ox + Rc) * S + (R.oy + Rc)) * (S + 1), z0 = Rc - R.zpe, z1 = Rc + R.zpe;
+            for (int z = z0 & ~1; z <= z1; z += 2) {
+                const bool a = z >= z0, b = z + 1 <= z1;
+                B.duo.push_back((c0 + z) << 2 | (int)a | (int)b << 1);
+                B.duo_k.push_back(a ? R.pe_start + z - z0 : -1);
+                B.duo_k.push_back(b ? R.pe_start + z + 1 - z0 : -1);
+            }
+        }
+    B.layer.clear();
+    B.layer_ir.clear();
+    for (int row = 0; row < (int)B.rows_me.size(); ++row) {
+        const RowRec& R = B.rows_me[row];
+        for (int z = R.zpe + 1; z <= std::min<int>(R.zn, R.zme); ++z) {
+            const double x = R.ox * delta[0], y = R.oy * delta[1], zz = z * delta[2];
+            B.layer.push_back(row << 8 | z);
+            B.layer_ir.push_back(1.0 / std::sqrt(x * x + y * y + zz * zz));
+        }
+    }
+}
+
 bool build_cluster_layout(const HostBall& B, int C, ClusterLayout& L, std::vector<int>& pt_slab, bool pitch4,
                           int max_planes) {
     const int R = B.r_pe, P = 2 * R + 1;
@@ -731,33 +768,10 @@ static bool build_march_groups(const HostBall& B, const std::vector<HostMGLevel>
     return true;
 }
 
-bool build_march(const HostBall& B, const std::vector<HostMGLevel>& levels, const double delta[3], int threads,
-                 HostMarch& H) {
+bool build_march(const HostBall& B, const std::vector<HostMGLevel>& levels, int threads, HostMarch& H) {
     for (int groups = 8; groups >= 1; --groups) {  // as many as fit the shared memory of an SM
         if (!build_march_groups(B, levels, threads, groups, H)) return false;
-        if (H.G.smem_floats > 55 * 1024) continue;
-        // the rim, and the shell layer with its 1 / r
-        H.rim.clear();
-        const int in2 = B.r_pe > 3 ? (B.r_pe - 3) * (B.r_pe - 3) : -1;
-        for (int pass = 0; pass < 2; ++pass) {
-            for (int k = 0; k < B.n_pe; ++k) {
-                const int x = (B.off[k] & 255) - 128, y = ((B.off[k] >> 8) & 255) - 128, z = ((B.off[k] >> 16) & 255) - 128;
-                if ((x * x + y * y + z * z > in2) == (pass == 0)) H.rim.push_back(k);
-            }
-            if (pass == 0) H.G.n_rim = (int)H.rim.size();
-        }
-        H.layer.clear();
-        H.layer_ir.clear();
-        for (int row = 0; row < (int)B.rows_me.size(); ++row) {
-            const RowRec& R = B.rows_me[row];
-            for (int z = R.zpe + 1; z <= std::min<int>(R.zn, R.zme); ++z) {
-                const double x = R.ox * delta[0], y = R.oy * delta[1], zz = z * delta[2];
-                H.layer.push_back(row << 8 | z);
-                H.layer_ir.push_back(1.0 / std::sqrt(x * x + y * y + zz * zz));
-            }
-        }
-        H.G.n_layer = (int)H.layer.size();
-        return true;
+        if (H.G.smem_floats <= 55 * 1024) return true;
     }
     return false;
 }

@@ -47,7 +47,20 @@ struct BallGeo {
     const int* sh_near;
     const int* sh_far;
     int n_near, n_far;
+    const int* rim;          // [n_pe] the PE points whose stencils reach the shell (n_rim), then the others
+    int n_rim;
+    // the near shell points again, z and -z as one: ME row << 8 | |z|, and 1 / r
+    const int* layer;
+    const double* layer_ir;
+    int n_layer;
+    // The PE points in pairs (z even and odd), by bands of kBand rows in y, then
+    // x, y, z: [n_duo] index of the first in a cube with rows of S + 1 (times 4;
+    // bits 0, 1: the points on the ball), [n_duo] the two's compact indices (-1: none)
+    const int* duo;
+    const int2* duo_k;
+    int n_duo;
 };
+constexpr int kBand = 12;
 
 // 19-point Laplacian coefficients of Eq. d2_1 on an orthorhombic grid:
 // lap f(c) = c0 f(c) + sum_a sum_q ca[q-1] (f(c + q s_a) + f(c - q s_a)).
@@ -116,12 +129,6 @@ struct MarchGeo {
     MarchLv lv[kMarchMax + 1];  // lv[nm]: only the columns of the first shared-memory level
     MarchSmall sl[kMGMax + 1];
     const int* qidx;            // [n_pe] index of each PE point in a level-0 vector
-    const int* rim;             // [n_pe] the PE points whose stencils reach the shell (n_rim), then the others
-    int n_rim;
-    // shell points that the stencil reads, z and -z as one: ME row << 8 | |z|, and 1 / r
-    const int* layer;
-    const double* layer_ir;
-    int n_layer;
 };
 
 // Everything the pair kernel needs, passed by value.

@@ -329,6 +329,233 @@ static __device__ __noinline__ void scatter_dxx(const SolveParams& P, const Ball
     }
 }
 
+// Step V scatter on full grids with FP64 adds (scatter_dxx has the other
+// forms): four points a turn, all their loads before the adds.
+static __device__ __noinline__ void scatter_wide(const SolveParams& P, const BallGeo& G, const PairRec& pr,
+                                                 const double* __restrict__ vc, int tid, int nthr) {
+    if (!P.dxx || P.box_org || P.dfix != 0.0) {
+        scatter_dxx(P, G, pr, vc, tid, nthr);
+        return;
+    }
+    const long long ng = P.ostride;
+    const double* __restrict__ phi_i = P.phi + (long long)pr.i * ng;
+    const double* __restrict__ phi_j = P.phi + (long long)pr.j * ng;
+    double* Di = P.dxx + (long long)pr.i * ng;
+    double* Dj = P.dxx + (long long)pr.j * ng;
+    const bool two = pr.i != pr.j;
+    const int N[3] = {P.N[0], P.N[1], P.N[2]}, g[3] = {pr.g[0], pr.g[1], pr.g[2]};
+    const int n = G.n_me;
+    const int* __restrict__ off = G.pt_off;
+    const int* __restrict__ cube = G.pt_cube;
+    for (int q0 = tid; q0 < n; q0 += 4 * nthr) {
+        long long gi[4];
+        double v[4], a[4], b[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int q = q0 + u * nthr;
+            gi[u] = -1;
+            if (q < n) {
+                gi[u] = grid_index(N, g, __ldg(off + q));
+                v[u] = vc[__ldg(cube + q)];
+                b[u] = phi_j[gi[u]];
+                a[u] = two ? phi_i[gi[u]] : 0.0;
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+            if (gi[u] >= 0) {
+                atomicAdd(Di + gi[u], v[u] * b[u]);
+                if (two) atomicAdd(Dj + gi[u], v[u] * a[u]);
+            }
+    }
+}
+
+// Step III: rho on the PE ball, v = 0 there; this thread's largest |rho|. Four
+// points a turn: their eight loads from the orbitals are in flight together.
+template <bool BOX>
+static __device__ __noinline__ double gather_wide(const SolveParams& P, const BallGeo& G, const PairRec& pr,
+                                                  double* __restrict__ rho, double* __restrict__ vc, int tid, int nthr) {
+    const double* __restrict__ phi_i = P.phi + (long long)pr.i * P.ostride;
+    const double* __restrict__ phi_j = P.phi + (long long)pr.j * P.ostride;
+    const int N[3] = {P.N[0], P.N[1], P.N[2]}, g[3] = {pr.g[0], pr.g[1], pr.g[2]};
+    const int bd[3] = {P.bdim[0], P.bdim[1], P.bdim[2]};
+    const int i = pr.i, j = pr.j, n = G.n_pe;
+    const int* __restrict__ off = G.pt_off;
+    const int* __restrict__ cube = G.pt_cube;
+    double big = 0.0;
+    for (int k0 = tid; k0 < n; k0 += 4 * nthr) {
+        double a[4], b[4];
+        int c[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int k = k0 + u * nthr;
+            a[u] = b[u] = 0.0;
+            if (k < n) {
+                c[u] = __ldg(cube + k);
+                const int pk = __ldg(off + k);
+                if constexpr (BOX) {
+                    const long long ii = orb_index(N, g, pk, P.box_org, bd, i), ij = orb_index(N, g, pk, P.box_org, bd, j);
+                    if (ii >= 0 && ij >= 0) {
+                        a[u] = phi_i[ii];
+                        b[u] = phi_j[ij];
+                    }
+                } else {
+                    const long long gi = grid_index(N, g, pk);
+                    a[u] = phi_i[gi];
+                    b[u] = phi_j[gi];
+                }
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int k = k0 + u * nthr;
+            if (k < n) {
+                const double r = a[u] * b[u];
+                rho[k] = r;
+                vc[c[u]] = 0.0;
+                big = fmax(big, fabs(r));
+            }
+        }
+    }
+    return big;
+}
+
+// Eq. mepole, stage 1: row sums S_c = sum_z z^c rho, c <= 6, a row per thread,
+// z and -z together: rho(z) +- rho(-z) feed the even and the odd c, 9 FP64
+// operations per two points (14 one by one; the FP64 pipe bounds this).
+static __device__ __noinline__ void moment_rows_folded(const SolveParams& P, const BallGeo& G,
+                                                       const double* __restrict__ rho, double* __restrict__ rowS,
+                                                       int tid, int nthr) {
+    const RowRec* __restrict__ rows = G.rows_pe;
+    const double* __restrict__ zp = P.pow_tab + (size_t)(2 * (2 * P.Rc + 1) + P.Rc) * 8;  // z = 0
+    for (int row = tid; row < G.n_rows_pe; row += nthr) {
+        const RowRec R = rows[row];
+        const double* rr = rho + R.pe_start + R.zpe;
+        double s0 = rr[0], s1 = 0.0, s2 = 0.0, s3 = 0.0, s4 = 0.0, s5 = 0.0, s6 = 0.0;
+#pragma unroll 2
+        for (int z = 1; z <= R.zpe; ++z) {
+            const double* __restrict__ w = zp + 8 * z;
+            const double p = rr[z], m = rr[-z];
+            const double e = p + m, o = p - m;
+            s0 += e;
+            s1 = fma(o, __ldg(w + 1), s1);
+            s2 = fma(e, __ldg(w + 2), s2);
+            s3 = fma(o, __ldg(w + 3), s3);
+            s4 = fma(e, __ldg(w + 4), s4);
+            s5 = fma(o, __ldg(w + 5), s5);
+            s6 = fma(e, __ldg(w + 6), s6);
+        }
+        double* o = rowS + 8 * row;
+        o[0] = s0;
+        o[1] = s1;
+        o[2] = s2;
+        o[3] = s3;
+        o[4] = s4;
+        o[5] = s5;
+        o[6] = s6;
+    }
+}
+
+// Eq. me on the shell. Per x plane the products V = T x^a of every monomial;
+// per ME row the coefficients U_{l,c} of P_l(z), polynomials in y (Horner, 56
+// FP64 operations a row; 168 term by term), u-major so that a warp shares u;
+// then the points. The boundary layer that the stencil reads is evaluated in
+// FP64, z and -z together: the even and odd parts of the P_l share the powers
+// of 1 / r^2, and 1 / r of every layer point comes from a table of the ball (33
+// FP64 operations for two points; 86 one by one with the root). The rest of
+// the shell only feeds D_xx: FP32, from the FP32 copy of U. Returns this
+// thread's largest |v| on the layer.
+static __device__ __noinline__ void shell_planes(const SolveParams& P, const BallGeo& G, const double* __restrict__ T,
+                                                 double* __restrict__ V, int tid, int nthr) {
+    const int Rc = P.Rc, np = 2 * G.r_me + 1;
+    const double* __restrict__ xp = P.pow_tab;
+    for (int it = tid; it < np * kNMono; it += nthr) {
+        const int pl = it / kNMono, m = it - pl * kNMono;
+        V[it] = T[m] * __ldg(xp + (pl - G.r_me + Rc) * 8 + c_mp.mono[m][0]);
+    }
+}
+
+static __device__ __noinline__ void shell_coeffs(const SolveParams& P, const BallGeo& G, const double* __restrict__ V,
+                                                 double* __restrict__ U64, float* __restrict__ U32, int tid, int nthr) {
+    const int nr = G.n_rows_me, Rc = P.Rc;
+    const double* __restrict__ yp = P.pow_tab + (2 * Rc + 1) * 8;
+    const RowRec* __restrict__ rows = G.rows_me;
+#pragma unroll 1
+    for (int l = 0; l <= kLmaxMax; ++l)
+#pragma unroll 1
+        for (int c = 0; c <= l; ++c) {
+            const int u = l * (l + 1) / 2 + c, m0 = l * (l + 1) * (l + 2) / 6 + c;
+            for (int row = tid; row < nr; row += nthr) {
+                const RowRec R = rows[row];
+                const double* __restrict__ v = V + (R.ox + G.r_me) * kNMono + m0;
+                const double y = __ldg(yp + (R.oy + Rc) * 8 + 1);
+                double acc = v[l * (l + 1) / 2];  // b = l - c
+                for (int q = l - 1; q >= c; --q) acc = fma(acc, y, v[q * (q + 1) / 2]);
+                U64[u * nr + row] = acc;
+                U32[u * nr + row] = (float)acc;
+            }
+        }
+}
+
+static __device__ __noinline__ double shell_values(const SolveParams& P, const BallGeo& G, const double* __restrict__ U64,
+                                                   const float* __restrict__ U32, double* __restrict__ vc, int tid,
+                                                   int nthr) {
+    const int nr = G.n_rows_me, Rc = P.Rc;
+    const RowRec* __restrict__ rows = G.rows_me;
+    const double dx = P.delta[0], dy = P.delta[1], dz = P.delta[2];
+    const long long S2 = P.S2, side = P.S;
+    double big = 0.0;
+    for (int q = tid; q < G.n_layer; q += nthr) {
+        const int pk = __ldg(G.layer + q), row = pk >> 8, z = pk & 255;
+        const double ir = __ldg(G.layer_ir + q);
+        const RowRec R = rows[row];
+        const double* __restrict__ U = U64 + row;
+        const double zz = z * dz, z2 = zz * zz, ir2 = ir * ir;
+        double e = 0.0, o = 0.0;
+#pragma unroll
+        for (int l = kLmaxMax; l >= 0; --l) {
+            const double* __restrict__ Ul = U + (size_t)(l * (l + 1) / 2) * nr;
+            double pe = Ul[(size_t)(l & ~1) * nr];
+#pragma unroll
+            for (int c = (l & ~1) - 2; c >= 0; c -= 2) pe = fma(pe, z2, Ul[(size_t)c * nr]);
+            e = l == kLmaxMax ? pe : fma(e, ir2, pe);
+            if (l >= 1) {
+                const int c0 = ((l - 1) & ~1) + 1;
+                double po = Ul[(size_t)c0 * nr];
+#pragma unroll
+                for (int c = c0 - 2; c >= 1; c -= 2) po = fma(po, z2, Ul[(size_t)c * nr]);
+                o = l == kLmaxMax ? po : fma(o, ir2, po);
+            } else {
+                o = o * ir2;
+            }
+        }
+        o *= zz;
+        const long long base = (long long)(R.ox + Rc) * S2 + (long long)(R.oy + Rc) * side + Rc;
+        const double vp = (e + o) * ir, vm = (e - o) * ir;
+        vc[base + z] = vp;
+        vc[base - z] = vm;  // z = 0: o = 0
+        big = fmax(big, fmax(fabs(vp), fabs(vm)));
+    }
+    for (int q = tid; q < G.n_far; q += nthr) {
+        const int pk = __ldg(G.sh_far + q), row = pk >> 8, z = (pk & 255) - 128;
+        const RowRec R = rows[row];
+        const float* __restrict__ U = U32 + row;
+        const float x = R.ox * (float)dx, y = R.oy * (float)dy, zz = (float)z * (float)dz;
+        const float ir = rsqrtf(fmaf(zz, zz, fmaf(x, x, y * y))), ir2 = ir * ir;
+        float acc = 0.0f;
+#pragma unroll
+        for (int l = kLmaxMax; l >= 0; --l) {
+            const float* __restrict__ Ul = U + (size_t)(l * (l + 1) / 2) * nr;
+            float pl = Ul[(size_t)l * nr];
+#pragma unroll
+            for (int c = l - 1; c >= 0; --c) pl = fmaf(pl, zz, Ul[(size_t)c * nr]);
+            acc = fmaf(acc, ir2, pl);
+        }
+        vc[(long long)(R.ox + Rc) * S2 + (long long)(R.oy + Rc) * side + Rc + z] = (double)(acc * ir);
+    }
+    return big;
+}
+
 __device__ __forceinline__ Stencil<double> negated(const Stencil<double>& s) {
     Stencil<double> n;
     n.c0 = -s.c0;

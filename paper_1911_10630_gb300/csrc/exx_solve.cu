@@ -384,12 +384,6 @@ size_t pair_kernel_smem(int Rc, int r_pe_max) {
     return sizeof(double) * ((size_t)3 * (2 * Rc + 1) * 8 + (size_t)(2 * r_pe_max + 1) * 28);
 }
 
-template <int NT, bool MIXED>
-static cudaError_t launch_t(const SolveParams& P, int grid, size_t smem, cudaStream_t st) {
-    pair_kernel<NT, MIXED><<<grid, NT, smem, st>>>(P);
-    return cudaGetLastError();
-}
-
 cudaError_t launch_pair_kernel(const SolveParams& P, int threads, bool mixed, int grid, size_t smem, cudaStream_t st) {
     if (P.mg) {  // the multigrid-preconditioned CG: FP64, or FP32 inside FP64 refinement
         if (!mixed) pair_kernel<512, false, true><<<grid, 512, smem, st>>>(P);
@@ -399,10 +393,11 @@ cudaError_t launch_pair_kernel(const SolveParams& P, int threads, bool mixed, in
         else pair_kernel<512, true, true><<<grid, 512, smem, st>>>(P);
         return cudaGetLastError();
     }
-    if (threads == 256) return mixed ? launch_t<256, true>(P, grid, smem, st) : launch_t<256, false>(P, grid, smem, st);
-    if (threads == 1024)
-        return mixed ? launch_t<1024, true>(P, grid, smem, st) : launch_t<1024, false>(P, grid, smem, st);
-    return mixed ? launch_t<512, true>(P, grid, smem, st) : launch_t<512, false>(P, grid, smem, st);
+    // without a hierarchy: FP32 inside FP64 refinement (FP64: exx_cg64.cu)
+    if (threads == 256) pair_kernel<256, true><<<grid, 256, smem, st>>>(P);
+    else if (threads == 1024) pair_kernel<1024, true><<<grid, 1024, smem, st>>>(P);
+    else pair_kernel<512, true><<<grid, 512, smem, st>>>(P);
+    return cudaGetLastError();
 }
 
 cudaError_t pair_kernel_occupancy(int threads, bool mixed, bool mg, bool one_ball, size_t smem, int* blocks_per_sm) {
@@ -412,9 +407,9 @@ cudaError_t pair_kernel_occupancy(int threads, bool mixed, bool mg, bool one_bal
     else if (mg && threads == 256) f = (const void*)pair_kernel<256, true, true>;
     else if (mg && threads == 1024) f = (const void*)pair_kernel<1024, true, true>;
     else if (mg) f = (const void*)pair_kernel<512, true, true>;
-    else if (threads == 256) f = mixed ? (const void*)pair_kernel<256, true> : (const void*)pair_kernel<256, false>;
-    else if (threads == 1024) f = mixed ? (const void*)pair_kernel<1024, true> : (const void*)pair_kernel<1024, false>;
-    else f = mixed ? (const void*)pair_kernel<512, true> : (const void*)pair_kernel<512, false>;
+    else if (threads == 256) f = (const void*)pair_kernel<256, true>;
+    else if (threads == 1024) f = (const void*)pair_kernel<1024, true>;
+    else f = (const void*)pair_kernel<512, true>;
     cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, f, threads, smem);
