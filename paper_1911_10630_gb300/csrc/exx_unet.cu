@@ -344,15 +344,32 @@ __global__ void head_backward_kernel(const float* __restrict__ in, const float* 
     }
 }
 
-// out[i] = sum over s = 0 .. n_parts - 1 of part[s * stride + i], in that order
-// (the fixed-order second stage of every gradient and loss reduction).
-__global__ void reduce_parts_kernel(const float* __restrict__ part, int n_parts, long long stride, int count,
-                                    float* __restrict__ out) {
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < count; i += gridDim.x * blockDim.x) {
-        float s = 0.0f;
-        for (int k = 0; k < n_parts; ++k) s += part[(size_t)k * stride + i];
-        out[i] = s;
+// out[i] = sum over s of part[s * stride + i], s < n_parts (the fixed-order
+// second stage of every gradient and loss reduction): 32 outputs to a block, 32
+// threads to an output, thread k adding the parts k, k + 32, ...; the 32 sums are
+// added in order. One thread per output left a chain of up to 2,432 loads (190 us;
+// 8 now, for the head's 18 values).
+__global__ void __launch_bounds__(1024) reduce_parts_kernel(const float* __restrict__ part, int n_parts,
+                                                            long long stride, int count, float* __restrict__ out) {
+    __shared__ float sum[32][33];
+    const int i = blockIdx.x * 32 + threadIdx.x;
+    float s = 0.0f;
+    if (i < count) {
+#pragma unroll 4
+        for (int k = threadIdx.y; k < n_parts; k += 32) s += __ldg(part + (size_t)k * stride + i);
     }
+    sum[threadIdx.y][threadIdx.x] = s;
+    __syncthreads();
+    if (threadIdx.y == 0 && i < count) {
+        float t = 0.0f;
+#pragma unroll
+        for (int k = 0; k < 32; ++k) t += sum[k][threadIdx.x];
+        out[i] = t;
+    }
+}
+cudaError_t reduce_parts(const float* part, int n_parts, long long stride, int count, float* out, cudaStream_t st) {
+    reduce_parts_kernel<<<(count + 31) / 32, dim3(32, 32), 0, st>>>(part, n_parts, stride, count, out);
+    return cudaGetLastError();
 }
 
 // 2x2x2 average pooling, channels last; one thread per (coarse voxel, 8 channels).
@@ -572,34 +589,96 @@ __global__ void __launch_bounds__(kDwThreads) dw_kernel(const __nv_bfloat16* __r
     }
 }
 
-// Weight gradient of the FP32 input layer: 27 x kIn x 16 weights and 16
-// biases; voxels split over blocks, each block's partial sums in
-// part[block][27 * kIn * 16 + 16] (added in block order afterwards).
-__global__ void dw_first_kernel(const float* __restrict__ in, const __nv_bfloat16* __restrict__ g,
-                                float* __restrict__ part, int B, int S, int nsplit) {
-    constexpr int CI = kCin[0], NW = 27 * CI * 16;
-    const long long nv = (long long)B * S * S * S;
-    const long long per = (nv + nsplit - 1) / nsplit;
-    const long long v0 = blockIdx.x * per, v1 = v0 + per < nv ? v0 + per : nv;
-    for (int t = threadIdx.x; t < NW + 16; t += blockDim.x) {
-        float acc = 0.0f;
-        if (t < NW) {
-            const int tap = t / (CI * 16), ci = (t / 16) % CI, co = t % 16;
-            const int dz = tap / 9 - 1, dy = (tap / 3) % 3 - 1, dx = tap % 3 - 1;
-            for (long long v = v0; v < v1; ++v) {
-                const int xx = (int)(v % S), yy = (int)((v / S) % S), zz = (int)((v / ((long long)S * S)) % S);
-                const long long bb = v / ((long long)S * S * S);
-                const int z2 = zz + dz, y2 = yy + dy, x2 = xx + dx;
-                if (z2 < 0 || z2 >= S || y2 < 0 || y2 >= S || x2 < 0 || x2 >= S) continue;
-                const long long u = ((bb * S + z2) * S + y2) * S + x2;
-                acc = fmaf(in[CI * u + ci], bf2f(g[v * 16 + co]), acc);
-            }
-        } else {
-            const int co = t - NW;
-            for (long long v = v0; v < v1; ++v) acc += bf2f(g[v * 16 + co]);
+// Weight gradient of the FP32 input layer: 27 x kIn x 16 weights and 16 biases,
+// with dw_kernel's voxel tiles. A block stages a tile (the halo of in and the tile
+// of g) and 4 groups of 81 threads (tap, ci) take 4 of its 16 rows each, 16 FMAs
+// to one value of in and a broadcast row of g; 16 more threads add g up. Split s
+// takes the tiles [s T / nsplit, (s + 1) T / nsplit); the groups' sums are added in
+// order into part[s][27 kIn 16 + 16]. One thread per weight running over the
+// voxels, its indices divided out of each, took 10.2 ms on a batch of 32 cubes of
+// 32; this 0.2.
+constexpr int kDwFirstTap = 27 * kIn, kDwFirstGroups = 4;
+constexpr int kDwFirstThreads = (kDwFirstTap * kDwFirstGroups + 16 + 31) / 32 * 32;
+
+__global__ void __launch_bounds__(kDwFirstThreads) dw_first_kernel(const float* __restrict__ in,
+                                                                   const __nv_bfloat16* __restrict__ g,
+                                                                   float* __restrict__ part, int B, int S, int nsplit) {
+    constexpr int CI = kIn, NW = 27 * CI * 16, HW = kDwHW * CI;
+    __shared__ float xs[kDwHD * kDwHH * HW];
+    __shared__ __align__(16) float gs[kDwVox][16];
+    __shared__ float sum[kDwFirstTap][17];
+    const int tid = threadIdx.x;
+    const int group = tid / kDwFirstTap, w = tid - group * kDwFirstTap;
+    const int tap = w / CI, ci = w - tap * CI;
+    const int dz = tap / 9, dy = (tap / 3) % 3, dx = tap % 3;
+    const bool acc_thread = group < kDwFirstGroups;
+    const int bias = tid - kDwFirstTap * kDwFirstGroups;  // 0 .. 15: adds g
+    const int td = (S + kDwD - 1) / kDwD, th = (S + kDwH - 1) / kDwH, tw = (S + kDwW - 1) / kDwW;
+    const long long T = (long long)B * td * th * tw;
+    const long long t0 = T * blockIdx.x / nsplit, t1 = T * (blockIdx.x + 1) / nsplit;
+    float acc[16], bacc = 0.0f;
+#pragma unroll
+    for (int k = 0; k < 16; ++k) acc[k] = 0.0f;
+    for (long long t = t0; t < t1; ++t) {
+        long long r = t;
+        const int w0 = (int)(r % tw) * kDwW;
+        r /= tw;
+        const int h0 = (int)(r % th) * kDwH;
+        r /= th;
+        const int d0 = (int)(r % td) * kDwD;
+        const int b = (int)(r / td);
+        __syncthreads();  // the previous tile's values are no longer read
+        for (int u = tid; u < kDwHD * kDwHH * HW; u += kDwFirstThreads) {
+            const int row = u / HW, e = u - row * HW;
+            const int d = d0 - 1 + row / kDwHH, h = h0 - 1 + row % kDwHH, x = w0 - 1 + e / CI;
+            const bool live = d >= 0 && d < S && h >= 0 && h < S && x >= 0 && x < S;
+            xs[u] = live ? in[((((long long)b * S + d) * S + h) * S + x) * CI + e % CI] : 0.0f;
         }
-        part[(size_t)blockIdx.x * (NW + 16) + t] = acc;
+        for (int u = tid; u < 2 * kDwVox; u += kDwFirstThreads) {
+            const int half = u & 1, vx = u >> 1;
+            const int d = d0 + vx / (kDwH * kDwW), h = h0 + (vx / kDwW) % kDwH, x = w0 + vx % kDwW;
+            uint4 q = make_uint4(0u, 0u, 0u, 0u);
+            if (d < S && h < S && x < S)
+                q = *reinterpret_cast<const uint4*>(g + ((((long long)b * S + d) * S + h) * S + x) * 16 + half * 8);
+            const __nv_bfloat16* qb = reinterpret_cast<const __nv_bfloat16*>(&q);
+#pragma unroll
+            for (int e = 0; e < 8; ++e) gs[vx][half * 8 + e] = bf2f(qb[e]);
+        }
+        __syncthreads();
+        if (acc_thread) {
+#pragma unroll
+            for (int q = 0; q < kDwD * kDwH / kDwFirstGroups; ++q) {
+                const int row = group + q * kDwFirstGroups, vd = row / kDwH, vh = row % kDwH;
+                const float* xrow = xs + ((vd + dz) * kDwHH + vh + dy) * HW + dx * CI + ci;
+                const float4* grow = reinterpret_cast<const float4*>(gs[row * kDwW]);
+#pragma unroll
+                for (int vw = 0; vw < kDwW; ++vw) {
+                    const float xv = xrow[vw * CI];
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) {
+                        const float4 gq = grow[vw * 4 + k];
+                        acc[4 * k + 0] = fmaf(xv, gq.x, acc[4 * k + 0]);
+                        acc[4 * k + 1] = fmaf(xv, gq.y, acc[4 * k + 1]);
+                        acc[4 * k + 2] = fmaf(xv, gq.z, acc[4 * k + 2]);
+                        acc[4 * k + 3] = fmaf(xv, gq.w, acc[4 * k + 3]);
+                    }
+                }
+            }
+        } else if (bias < 16) {
+            for (int vx = 0; vx < kDwVox; ++vx) bacc += gs[vx][bias];
+        }
     }
+    float* dw = part + (size_t)blockIdx.x * (NW + 16);
+    for (int q = 0; q < kDwFirstGroups; ++q) {
+        __syncthreads();
+        if (acc_thread && group == q) {
+#pragma unroll
+            for (int k = 0; k < 16; ++k) sum[w][k] = q ? sum[w][k] + acc[k] : acc[k];
+        }
+    }
+    __syncthreads();
+    for (int u = tid; u < NW; u += kDwFirstThreads) dw[u] = sum[u / 16][u % 16];
+    if (!acc_thread && bias < 16) dw[NW + bias] = bacc;
 }
 
 __global__ void adam_kernel(float* __restrict__ p, const float* __restrict__ g, float* __restrict__ m,
@@ -867,8 +946,8 @@ cudaError_t backward(Net& n, const float* in, const float* target, int B, cudaSt
         float* ghw = n.grads + param_offset(kHead);
         head_backward_kernel<<<nblk, 256, 0, st>>>(in, target, n.out, n.y0, n.params + param_offset(kHead), n.g_y0,
                                                    n.gpart, v0, 1.0f / (float)v0);
-        reduce_parts_kernel<<<1, 32, 0, st>>>(n.gpart, nblk, 18, 17, ghw);
-        reduce_parts_kernel<<<1, 32, 0, st>>>(n.gpart + 17, nblk, 18, 1, n.d_loss);
+        UCK(reduce_parts(n.gpart, nblk, 18, 17, ghw, st));
+        UCK(reduce_parts(n.gpart + 17, nblk, 18, 1, n.d_loss, st));
     }
     UCK(cudaGetLastError());
     // data gradient through layer l: from g (cout channels) to cin channels,
@@ -882,9 +961,8 @@ cudaError_t backward(Net& n, const float* in, const float* target, int B, cudaSt
         dim3 grid(nsplit, kCin[l] / 16, kCout[l] / 16);
         const int count = 27 * kCin[l] * kCout[l] + kCout[l];
         dw_kernel<<<grid, kDwThreads, 0, st>>>(x, g, n.gpart, B, s, kCin[l], kCout[l], nsplit);
-        reduce_parts_kernel<<<grid_for(count, n.n_sm), 256, 0, st>>>(n.gpart, nsplit, count, count,
-                                                                     n.grads + param_offset(l));
-        return cudaGetLastError();
+        UCK(cudaGetLastError());
+        return reduce_parts(n.gpart, nsplit, count, count, n.grads + param_offset(l), st);
     };
     // level 0, up path
     UCK(dweight(n.y0a, n.g_y0, 13, S));
@@ -928,9 +1006,9 @@ cudaError_t backward(Net& n, const float* in, const float* target, int B, cudaSt
     {
         const int nsplit = 4 * n.n_sm;
         const int count = 27 * kIn * 16 + 16;
-        dw_first_kernel<<<nsplit, 256, 0, st>>>(in, n.g_x0a, n.gpart, B, S, nsplit);
-        reduce_parts_kernel<<<grid_for(count, n.n_sm), 256, 0, st>>>(n.gpart, nsplit, count, count,
-                                                                     n.grads + param_offset(0));
+        dw_first_kernel<<<nsplit, kDwFirstThreads, 0, st>>>(in, n.g_x0a, n.gpart, B, S, nsplit);
+        UCK(cudaGetLastError());
+        UCK(reduce_parts(n.gpart, nsplit, count, count, n.grads + param_offset(0), st));
     }
     return cudaGetLastError();
 }
