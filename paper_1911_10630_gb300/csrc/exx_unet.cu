@@ -35,165 +35,275 @@ constexpr int kWaitLimit = 1 << 22;
 __device__ __forceinline__ float bf2f(__nv_bfloat16 v) { return __bfloat162float(v); }
 __device__ __forceinline__ __nv_bfloat16 f2bf(float v) { return __float2bfloat16_rn(v); }
 
+constexpr int kStages = 4;
 struct ConvArgs {
     const __nv_bfloat16* x;
+    const __nv_bfloat16* low;  // the first cl input channels come from here, at half the resolution (cl = 0: none)
     const __nv_bfloat16* wp;
     const float* bias;
     const __nv_bfloat16* mask;
     __nv_bfloat16* y;
-    int B, D, H, W, cin, cout;
-    int epi, DT, ncols, nbuf;
+    int B, D, H, W, cin, cl, cout;
+    int nb, nsplit;  // output channels per tile: nb of cout, nsplit slices
+    int epi, DT, ncols, acc_cols, n_acc, n_stage;
     int fold;  // the three depth taps of a (dh, dw) in one MMA of N = 3 cout (depth-shifted TMEM slices)
-    int tiles_d, tiles_h, tiles_w;
+    int tiles_d, tiles_h, tiles_w, n_tiles;
+    int resident;  // all weights stay in shared memory
     uint32_t itile, wtile, stage;
     int* err;
 };
 
-__global__ void __launch_bounds__(128) conv3_tc_kernel(const ConvArgs a) {
+// Persistent CTAs, one per SM, each over the tiles t, t + grid, ...: warps 0-3
+// empty the accumulators (epilogue), one thread of warp 4 issues the MMAs, warps
+// 5-12 stage the input halo tiles and weights. A unit is one 16-channel chunk of a
+// tile; units pass through n_stage shared-memory stages (full / empty barriers),
+// tiles through n_acc accumulators in tensor memory. One CTA per tile that staged,
+// multiplied and stored in turn left the tensor cores 5 to 10 % busy: the 13
+// convolutions of 32 cubes of 48 took 2.36 ms; with cheaper staging and two CTAs a
+// SM 1.2; like this 0.93.
+constexpr int kProducers = 256, kConvThreads = 5 * 32 + kProducers;
+
+__global__ void __launch_bounds__(kConvThreads, 1) conv3_tc_kernel(const __grid_constant__ ConvArgs a) {
     extern __shared__ unsigned char smem_dyn[];
-    __shared__ uint64_t mbar[2];
+    __shared__ uint64_t full[kStages], empty[kStages], acc_full[2], acc_empty[2], wres;
     __shared__ uint32_t s_tmem;
+    __shared__ float s_bias[256];
     unsigned char* base =
         reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_dyn) + 127) & ~uintptr_t(127));
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    int t = blockIdx.x;
-    const int tw = t % a.tiles_w;
-    t /= a.tiles_w;
-    const int th = t % a.tiles_h;
-    t /= a.tiles_h;
-    const int td = t % a.tiles_d;
-    const int b = t / a.tiles_d;
-    const int DT = a.DT;
-    const int d0 = td * DT, h0 = th * kTH, w0 = tw * kTW;
-
+    const int DT = a.DT, nch = a.cin / 16, NS = a.n_stage, NA = a.n_acc;
     if (tid == 0) {
-        tc::mbar_init(&mbar[0], 1);
-        tc::mbar_init(&mbar[1], 1);
+        for (int s = 0; s < kStages; ++s) {
+            tc::mbar_init(&full[s], kProducers / 32 + (a.resident ? 0 : 1));
+            tc::mbar_init(&empty[s], 1);
+        }
+        for (int s = 0; s < 2; ++s) {
+            tc::mbar_init(&acc_full[s], 1);
+            tc::mbar_init(&acc_empty[s], 128);
+        }
+        tc::mbar_init(&wres, 1);
         tc::mbar_init_fence();
     }
+    for (int i = tid; i < a.cout; i += kConvThreads) s_bias[i] = a.bias ? a.bias[i] : 0.0f;
     if (warp == 0) tc::tmem_alloc(&s_tmem, (uint32_t)a.ncols);
     tc::fence_before_sync();
     __syncthreads();
     tc::fence_after_sync();
     const uint32_t tbase = s_tmem;
     if (a.fold) {  // every slice accumulates from several MMAs: start from zero
-        for (int c0 = 0; c0 < a.ncols; c0 += 16) tc::tmem_st16_zero(tbase + ((uint32_t)(warp * 32) << 16) + c0);
-        tc::tmem_wait_st();
+        if (warp < 4) {
+            for (int c0 = 0; c0 < a.ncols; c0 += 16) tc::tmem_st16_zero(tbase + ((uint32_t)(warp * 32) << 16) + c0);
+            tc::tmem_wait_st();
+        }
         tc::fence_before_sync();
         __syncthreads();
         tc::fence_after_sync();
     }
-
-    const int nch = a.cin / 16;
-    const uint32_t idesc = tc::idesc_bf16_f32(128, a.fold ? 3 * a.cout : a.cout);
-    const int nvox = (DT + 2) * kHH * kWW;
+    unsigned char* stages = base + (a.resident ? (size_t)nch * a.wtile : 0);
+    // tile t: w fastest, then h, d, sample, slice of the output channels
+    const auto place = [&](int t, int& b, int& d0, int& h0, int& w0, int& n0) {
+        w0 = t % a.tiles_w * kTW;
+        t /= a.tiles_w;
+        h0 = t % a.tiles_h * kTH;
+        t /= a.tiles_h;
+        d0 = t % a.tiles_d * DT;
+        t /= a.tiles_d;
+        b = t % a.B;
+        n0 = t / a.B * a.nb;
+    };
     bool ok = true;
-    for (int c = 0; c < nch; ++c) {
-        const int s = a.nbuf == 2 ? (c & 1) : 0;
-        unsigned char* st = base + (size_t)s * a.stage;
-        if (c >= a.nbuf) {  // the MMAs of chunk c - nbuf read this buffer
-            const int prev = c - a.nbuf;
-            if (!tc::mbar_wait(&mbar[s], (uint32_t)((prev / a.nbuf) & 1), kWaitLimit)) ok = false;
+    if (warp >= 5) {  // staging
+        const int pt = tid - 5 * 32, items = (DT + 2) * kHH * kWW * 2;
+        const bool delay = NS >= 3;
+        const auto finish = [&](int s) {
+            tc::fence_proxy_async();
+            __syncwarp();
+            if (lane == 0) tc::mbar_arrive(&full[s]);
+        };
+        if (a.resident && pt == 0) {
+            tc::mbar_expect(&wres, (uint32_t)nch * a.wtile);
+            for (int c = 0; c < nch; ++c)
+                tc::bulk_load(base + (size_t)c * a.wtile, reinterpret_cast<const unsigned char*>(a.wp) + (size_t)c * a.wtile,
+                              a.wtile, &wres);
         }
-        if (!__syncthreads_and(ok)) {
-            ok = false;
-            break;
-        }
-        // input halo tile: two channel octets, [DT+2][18][10] voxels x 16 B each
-        for (int u = tid; u < 2 * nvox; u += 128) {
-            const int o = u >= nvox ? 1 : 0;
-            const int vx = u - o * nvox;
-            const int wx = vx % kWW, r2 = vx / kWW, hy = r2 % kHH, dz = r2 / kHH;
-            const int d = d0 - 1 + dz, h = h0 - 1 + hy, w = w0 - 1 + wx;
-            const bool in = d >= 0 && d < a.D && h >= 0 && h < a.H && w >= 0 && w < a.W;
-            const __nv_bfloat16* src =
-                in ? a.x + ((((size_t)b * a.D + d) * a.H + h) * a.W + w) * a.cin + c * 16 + o * 8 : a.x;
-            tc::cp_async16(st + (size_t)o * a.itile + (size_t)vx * 16, src, in ? 16u : 0u);
-        }
-        // weights of chunk c: [27][cout/8][2][8][8] BF16, contiguous
-        const unsigned char* wsrc = reinterpret_cast<const unsigned char*>(a.wp) + (size_t)c * a.wtile;
-        unsigned char* wdst = st + 2 * (size_t)a.itile;
-        for (uint32_t u = tid; u < a.wtile / 16; u += 128) tc::cp_async16(wdst + u * 16, wsrc + u * 16, 16u);
-        tc::cp_async_wait_all();
-        tc::fence_proxy_async();
-        __syncthreads();
-        if (tid == 0) {
-            tc::fence_after_sync();
-            const uint32_t sa = tc::smem_addr(st), sw = tc::smem_addr(wdst);
-            if (a.fold) {
-                // input slice u (depth d0 - 1 + u) feeds the outputs tt = u - dz,
-                // dz = 2, 1, 0: TMEM slices u .. u + 2 (slice = tt + 2), with the
-                // weights of (dh, dw) packed as three N-blocks in that order
-                for (int u = 0; u < DT + 2; ++u) {
-#pragma unroll 1
-                    for (int hw = 0; hw < 9; ++hw) {
-                        const int dh = hw / 3, dw = hw % 3;
-                        const uint32_t aoff = (uint32_t)(((u * kHH + dh) * kWW + dw) * 16);
-                        const uint64_t ad = tc::sdesc(sa + aoff, a.itile, kWW * 16);
-                        const uint64_t bd = tc::sdesc(sw + (uint32_t)(hw * 3 * a.cout * 32), 128, 256);
-                        tc::mma_bf16(tbase + (uint32_t)(u * a.cout), ad, bd, idesc, 1u);
+        int s = 0, k = 0, before = 0;
+        uint32_t ph = 1;  // parity of the stage's last release
+        for (int t = blockIdx.x; t < a.n_tiles && ok; t += gridDim.x) {
+            int b, d0, h0, w0, n0;
+            place(t, b, d0, h0, w0, n0);
+            for (int c = 0; c < nch; ++c, ++k) {
+                if (k >= NS) {
+                    ok = __all_sync(0xffffffffu, tc::mbar_wait(&empty[s], ph, kWaitLimit));
+                    if (!ok) break;
+                }
+                unsigned char* st = stages + (size_t)s * a.stage;
+                if (!a.resident && pt == 0) {
+                    // weights of chunk c: [27][cout/8][2][8][8] BF16
+                    const unsigned char* src = reinterpret_cast<const unsigned char*>(a.wp) + (size_t)c * 27 * a.cout * 32;
+                    unsigned char* dst = st + 2 * (size_t)a.itile;
+                    tc::mbar_expect(&full[s], a.wtile);
+                    if (a.nsplit == 1) {
+                        tc::bulk_load(dst, src, a.wtile, &full[s]);
+                    } else {
+                        for (int tap = 0; tap < 27; ++tap)
+                            tc::bulk_load(dst + (size_t)tap * a.nb * 32, src + ((size_t)tap * a.cout + n0) * 32,
+                                          (uint32_t)a.nb * 32u, &full[s]);
                     }
                 }
-            } else {
-                for (int tt = 0; tt < DT; ++tt) {
-#pragma unroll 1
-                    for (int tap = 0; tap < 27; ++tap) {
-                        const int dd = tap / 9, dh = (tap / 3) % 3, dw = tap % 3;
-                        const uint32_t aoff = (uint32_t)((((tt + dd) * kHH + dh) * kWW + dw) * 16);
-                        const uint64_t ad = tc::sdesc(sa + aoff, a.itile, kWW * 16);
-                        const uint64_t bd = tc::sdesc(sw + (uint32_t)(tap * a.cout * 32), 128, 256);
-                        tc::mma_bf16(tbase + (uint32_t)(tt * a.cout), ad, bd, idesc, (c > 0 || tap > 0) ? 1u : 0u);
-                    }
+                // input halo tile: two channel octets, [DT+2][18][10] voxels x 16 B each
+                const bool lo = c * 16 < a.cl;
+                const int sh = lo ? 1 : 0, D = a.D >> sh, H = a.H >> sh, W = a.W >> sh;
+                const int ch = lo ? a.cl : a.cin - a.cl;
+                const __nv_bfloat16* xb =
+                    (lo ? a.low : a.x) + (size_t)b * D * H * W * ch + (lo ? c * 16 : c * 16 - a.cl);
+#pragma unroll 2
+                for (int u = pt; u < items; u += kProducers) {
+                    const int row = u / (2 * kWW), e = u - row * (2 * kWW), o = e & 1, wx = e >> 1;
+                    const int dz = row / kHH, hy = row - dz * kHH;
+                    const int d = d0 - 1 + dz, h = h0 - 1 + hy, w = w0 - 1 + wx;
+                    const bool in =
+                        (unsigned)d < (unsigned)a.D && (unsigned)h < (unsigned)a.H && (unsigned)w < (unsigned)a.W;
+                    const __nv_bfloat16* src =
+                        in ? xb + (size_t)(((d >> sh) * H + (h >> sh)) * W + (w >> sh)) * ch + o * 8 : a.x;
+                    tc::cp_async16(st + (size_t)o * a.itile + (size_t)(row * kWW + wx) * 16, src, in ? 16u : 0u);
+                }
+                tc::cp_async_commit();
+                if (!delay) {
+                    tc::cp_async_wait<0>();
+                    finish(s);
+                } else if (k > 0) {  // one unit behind: its loads ran while this one's were issued
+                    tc::cp_async_wait<1>();
+                    finish(before);
+                }
+                before = s;
+                if (++s == NS) {
+                    s = 0;
+                    ph ^= 1u;
                 }
             }
-            tc::commit(&mbar[s]);
         }
-    }
-    if (ok) {
-        const int last = nch - 1, s = a.nbuf == 2 ? (last & 1) : 0;
-        if (!tc::mbar_wait(&mbar[s], (uint32_t)((last / a.nbuf) & 1), kWaitLimit)) ok = false;
+        if (delay && k > 0) {
+            tc::cp_async_wait<0>();
+            finish(before);
+        }
+    } else if (warp == 4) {
+        if (lane == 0) {
+            const uint32_t idesc = tc::idesc_bf16_f32(128, a.fold ? 3 * a.nb : a.nb);
+            const uint32_t bs = (uint32_t)(a.fold ? 3 : 1) * a.nb * 2;  // 16-byte words of weights per MMA
+            if (a.resident && !tc::mbar_wait(&wres, 0, kWaitLimit)) ok = false;
+            int s = 0, i = 0;
+            uint32_t ph = 0;
+            for (int t = blockIdx.x; t < a.n_tiles && ok; t += gridDim.x, ++i) {
+                const int ab = NA == 2 ? i & 1 : 0;
+                if (i >= NA && !tc::mbar_wait(&acc_empty[ab], (uint32_t)((i / NA - 1) & 1), kWaitLimit)) {
+                    ok = false;
+                    break;
+                }
+                const uint32_t acc = tbase + (uint32_t)(ab * a.acc_cols);
+                for (int c = 0; c < nch; ++c) {
+                    if (!tc::mbar_wait(&full[s], ph, kWaitLimit)) {
+                        ok = false;
+                        break;
+                    }
+                    tc::fence_after_sync();
+                    unsigned char* st = stages + (size_t)s * a.stage;
+                    const uint64_t ad0 = tc::sdesc(tc::smem_addr(st), a.itile, kWW * 16);
+                    const uint64_t bd0 = tc::sdesc(
+                        tc::smem_addr(a.resident ? base + (size_t)c * a.wtile : st + 2 * (size_t)a.itile), 128, 256);
+                    if (a.fold) {
+                        // input slice u (depth d0 - 1 + u) feeds the outputs tt = u - dz,
+                        // dz = 2, 1, 0: TMEM slices u .. u + 2 (slice = tt + 2), with the
+                        // weights of (dh, dw) packed as three N-blocks in that order
+                        for (int u = 0; u < DT + 2; ++u) {
+                            const uint64_t ad = ad0 + (uint32_t)(u * kHH * kWW);
+#pragma unroll
+                            for (int hw = 0; hw < 9; ++hw)
+                                tc::mma_bf16(acc + (uint32_t)(u * a.nb), ad + (uint32_t)((hw / 3) * kWW + hw % 3),
+                                             bd0 + hw * bs, idesc, 1u);
+                        }
+                    } else {
+                        for (int tt = 0; tt < DT; ++tt) {
+#pragma unroll 1
+                            for (int dd = 0; dd < 3; ++dd) {
+                                const uint64_t ad = ad0 + (uint32_t)((tt + dd) * kHH * kWW), bd = bd0 + dd * 9 * bs;
+#pragma unroll
+                                for (int hw = 0; hw < 9; ++hw)
+                                    tc::mma_bf16(acc + (uint32_t)(tt * a.nb), ad + (uint32_t)((hw / 3) * kWW + hw % 3),
+                                                 bd + hw * bs, idesc, (c > 0 || dd > 0 || hw > 0) ? 1u : 0u);
+                            }
+                        }
+                    }
+                    tc::commit(&empty[s]);
+                    if (++s == NS) {
+                        s = 0;
+                        ph ^= 1u;
+                    }
+                }
+                if (ok) tc::commit(&acc_full[ab]);
+            }
+        }
+        __syncwarp();
+    } else {
+        const int m = warp * 32 + lane;  // accumulator row = TMEM lane
+        const uint32_t row = (uint32_t)(warp * 32) << 16;
+        int i = 0;
+        for (int t = blockIdx.x; t < a.n_tiles; t += gridDim.x, ++i) {
+            int b, d0, h0, w0, n0;
+            place(t, b, d0, h0, w0, n0);
+            const int ab = NA == 2 ? i & 1 : 0;
+            ok = __all_sync(0xffffffffu, tc::mbar_wait(&acc_full[ab], (uint32_t)((i / NA) & 1), kWaitLimit));
+            if (!ok) break;
+            tc::fence_after_sync();
+            const uint32_t acc = tbase + row + (uint32_t)(ab * a.acc_cols + (a.fold ? 2 * a.nb : 0));
+            const int h = h0 + (m >> 3), w = w0 + (m & 7);
+            for (int tt = 0; tt < DT; ++tt) {
+                const int d = d0 + tt;
+                const bool live = d < a.D && h < a.H && w < a.W;
+                const size_t vox = (((size_t)b * a.D + d) * a.H + h) * a.W + w;
+                for (int c0 = 0; c0 < a.nb; c0 += 16) {
+                    float v[16];
+                    __syncwarp();
+                    tc::tmem_ld16(acc + (uint32_t)(tt * a.nb + c0), v);
+                    if (a.fold) tc::tmem_st16_zero(acc + (uint32_t)(tt * a.nb + c0));
+                    if (!live) continue;
+                    const size_t at = vox * a.cout + n0 + c0;
+                    if (a.bias) {
+#pragma unroll
+                        for (int k = 0; k < 16; ++k) v[k] += s_bias[n0 + c0 + k];
+                    }
+                    if (a.epi == 1) {
+#pragma unroll
+                        for (int k = 0; k < 16; ++k) v[k] = fmaxf(v[k], 0.0f);
+                    } else if (a.epi == 2) {
+                        const uint4* mp = reinterpret_cast<const uint4*>(a.mask + at);
+                        uint4 mm[2] = {mp[0], mp[1]};
+                        const __nv_bfloat16* mb = reinterpret_cast<const __nv_bfloat16*>(mm);
+#pragma unroll
+                        for (int k = 0; k < 16; ++k) v[k] = bf2f(mb[k]) > 0.0f ? v[k] : 0.0f;
+                    }
+                    uint4 o[2];
+                    __nv_bfloat16* ob = reinterpret_cast<__nv_bfloat16*>(o);
+#pragma unroll
+                    for (int k = 0; k < 16; ++k) ob[k] = f2bf(v[k]);
+                    uint4* yp = reinterpret_cast<uint4*>(a.y + at);
+                    yp[0] = o[0];
+                    yp[1] = o[1];
+                }
+            }
+            __syncwarp();
+            if (a.fold) tc::tmem_wait_st();
+            tc::fence_before_sync();
+            tc::mbar_arrive(&acc_empty[ab]);
+        }
     }
     ok = __syncthreads_and(ok);
-    tc::fence_after_sync();
-    if (ok) {
-        const int m = warp * 32 + lane;  // accumulator row = TMEM lane
-        const int h = h0 + (m >> 3), w = w0 + (m & 7);
-        for (int tt = 0; tt < DT; ++tt) {
-            const int d = d0 + tt;
-            const bool live = d < a.D && h < a.H && w < a.W;
-            const size_t vox = (((size_t)b * a.D + d) * a.H + h) * a.W + w;
-            for (int c0 = 0; c0 < a.cout; c0 += 16) {
-                float v[16];
-                tc::tmem_ld16(tbase + ((uint32_t)(warp * 32) << 16) + (uint32_t)((tt + (a.fold ? 2 : 0)) * a.cout + c0),
-                              v);
-                if (!live) continue;
-                if (a.bias) {
-#pragma unroll
-                    for (int k = 0; k < 16; ++k) v[k] += a.bias[c0 + k];
-                }
-                if (a.epi == 1) {
-#pragma unroll
-                    for (int k = 0; k < 16; ++k) v[k] = fmaxf(v[k], 0.0f);
-                } else if (a.epi == 2) {
-                    const uint4* mp = reinterpret_cast<const uint4*>(a.mask + vox * a.cout + c0);
-                    uint4 mm[2] = {mp[0], mp[1]};
-                    const __nv_bfloat16* mb = reinterpret_cast<const __nv_bfloat16*>(mm);
-#pragma unroll
-                    for (int k = 0; k < 16; ++k) v[k] = bf2f(mb[k]) > 0.0f ? v[k] : 0.0f;
-                }
-                uint4 o[2];
-                __nv_bfloat16* ob = reinterpret_cast<__nv_bfloat16*>(o);
-#pragma unroll
-                for (int k = 0; k < 16; ++k) ob[k] = f2bf(v[k]);
-                uint4* yp = reinterpret_cast<uint4*>(a.y + vox * a.cout + c0);
-                yp[0] = o[0];
-                yp[1] = o[1];
-            }
-        }
-    } else if (tid == 0) {
+    if (!ok && tid == 0) {
         atomicExch(a.err, 1);
-        // let MMAs still in flight finish before the tensor memory goes back
-        tc::mbar_wait(&mbar[0], 0, 1024);
+        // let MMAs and copies still in flight finish before their memory goes back
+        for (int s = 0; s < kStages; ++s) {
+            tc::mbar_wait(&empty[s], 0, 256);
+            tc::mbar_wait(&full[s], 0, 256);
+        }
     }
     tc::fence_before_sync();
     __syncthreads();
@@ -233,40 +343,74 @@ __global__ void pack_kernel(const float* __restrict__ w, __nv_bfloat16* __restri
 
 // ---- CUDA-core layers ------------------------------------------------------
 
-// Input layer: kIn FP32 channels -> 16, ReLU. One thread per output voxel.
-__global__ void conv_first_kernel(const float* __restrict__ in, const float* __restrict__ w,
-                                  const float* __restrict__ bias, __nv_bfloat16* __restrict__ y, int B, int S) {
-    constexpr int CI = kCin[0];
-    __shared__ float ws[27 * CI * 16 + 16];
+// Input layer: kIn FP32 channels -> 16, ReLU; S a multiple of 4. A thread makes 4
+// voxels along x: a weight read from shared memory (broadcast) serves 4 FMAs and an
+// input 48, which leaves the FMAs as the bound (1,296 a voxel: 0.12 ms on 32 cubes
+// of 48; one voxel per thread took 0.42 ms, this 0.23).
+// W16: in is 16-byte aligned (a caller's need not be).
+template <bool W16>
+__global__ void __launch_bounds__(256, 2) conv_first_kernel(const float* __restrict__ in, const float* __restrict__ w,
+                                                         const float* __restrict__ bias, __nv_bfloat16* __restrict__ y,
+                                                         int B, int S) {
+    constexpr int CI = kIn;
+    __shared__ __align__(16) float ws[27 * CI * 16 + 16];
     for (int i = threadIdx.x; i < 27 * CI * 16; i += blockDim.x) ws[i] = w[i];
     if (threadIdx.x < 16) ws[27 * CI * 16 + threadIdx.x] = bias[threadIdx.x];
     __syncthreads();
-    const long long nv = (long long)B * S * S * S;
-    for (long long v = blockIdx.x * (long long)blockDim.x + threadIdx.x; v < nv;
-         v += (long long)gridDim.x * blockDim.x) {
-        const int x = (int)(v % S), yy = (int)((v / S) % S), z = (int)((v / ((long long)S * S)) % S);
-        const long long bb = v / ((long long)S * S * S);
-        float acc[16];
+    const int S4 = S / 4;
+    const long long nq = (long long)B * S * S * S4;
+    for (long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x; q < nq; q += (long long)gridDim.x * blockDim.x) {
+        const int x = (int)(q % S4) * 4;
+        const long long row = q / S4;  // (b S + z) S + y
+        const int yy = (int)(row % S), z = (int)((row / S) % S);
+        float acc[4][16];
 #pragma unroll
-        for (int c = 0; c < 16; ++c) acc[c] = ws[27 * CI * 16 + c];
-        for (int tap = 0; tap < 27; ++tap) {
-            const int zz = z + tap / 9 - 1, y2 = yy + (tap / 3) % 3 - 1, x2 = x + tap % 3 - 1;
-            if (zz < 0 || zz >= S || y2 < 0 || y2 >= S || x2 < 0 || x2 >= S) continue;
-            const float* iv = in + (((bb * S + zz) * S + y2) * S + x2) * CI;
+        for (int c = 0; c < 16; ++c)
 #pragma unroll
-            for (int ci = 0; ci < CI; ++ci) {
-                const float a = iv[ci];
+            for (int v = 0; v < 4; ++v) acc[v][c] = ws[27 * CI * 16 + c];
+#pragma unroll 1
+        for (int zy = 0; zy < 9; ++zy) {
+            const int dz = zy / 3 - 1, dy = zy % 3 - 1;
+            if (z + dz < 0 || z + dz >= S || yy + dy < 0 || yy + dy >= S) continue;
+            const float* iv = in + ((row + dz * S + dy) * S + x) * CI;
+            float a[6 * CI];  // voxels x - 1 .. x + 4
 #pragma unroll
-                for (int c = 0; c < 16; ++c) acc[c] = fmaf(a, ws[(tap * CI + ci) * 16 + c], acc[c]);
+            for (int k = 0; k < CI; ++k) {
+                float4 f;
+                if constexpr (W16) f = *reinterpret_cast<const float4*>(iv + 4 * k);
+                else f = make_float4(iv[4 * k], iv[4 * k + 1], iv[4 * k + 2], iv[4 * k + 3]);
+                a[CI + 4 * k] = f.x;
+                a[CI + 4 * k + 1] = f.y;
+                a[CI + 4 * k + 2] = f.z;
+                a[CI + 4 * k + 3] = f.w;
+                a[k] = x > 0 ? iv[k - CI] : 0.0f;
+                a[5 * CI + k] = x + 4 < S ? iv[4 * CI + k] : 0.0f;
             }
-        }
-        uint4 o[2];
-        __nv_bfloat16* ob = reinterpret_cast<__nv_bfloat16*>(o);
+            const float4* wr = reinterpret_cast<const float4*>(ws + zy * 3 * CI * 16);
 #pragma unroll
-        for (int c = 0; c < 16; ++c) ob[c] = f2bf(fmaxf(acc[c], 0.0f));
-        uint4* yp = reinterpret_cast<uint4*>(y + v * 16);
-        yp[0] = o[0];
-        yp[1] = o[1];
+            for (int e = 0; e < 3 * CI; ++e)  // (dx, ci)
+#pragma unroll
+                for (int c4 = 0; c4 < 4; ++c4) {
+                    const float4 f = wr[e * 4 + c4];
+#pragma unroll
+                    for (int v = 0; v < 4; ++v) {
+                        acc[v][4 * c4 + 0] = fmaf(a[v * CI + e], f.x, acc[v][4 * c4 + 0]);
+                        acc[v][4 * c4 + 1] = fmaf(a[v * CI + e], f.y, acc[v][4 * c4 + 1]);
+                        acc[v][4 * c4 + 2] = fmaf(a[v * CI + e], f.z, acc[v][4 * c4 + 2]);
+                        acc[v][4 * c4 + 3] = fmaf(a[v * CI + e], f.w, acc[v][4 * c4 + 3]);
+                    }
+                }
+        }
+        uint4* yp = reinterpret_cast<uint4*>(y + (row * S + x) * 16);
+#pragma unroll
+        for (int v = 0; v < 4; ++v) {
+            uint4 o[2];
+            __nv_bfloat16* ob = reinterpret_cast<__nv_bfloat16*>(o);
+#pragma unroll
+            for (int c = 0; c < 16; ++c) ob[c] = f2bf(fmaxf(acc[v][c], 0.0f));
+            yp[2 * v] = o[0];
+            yp[2 * v + 1] = o[1];
+        }
     }
 }
 
@@ -345,30 +489,34 @@ __global__ void head_backward_kernel(const float* __restrict__ in, const float* 
 }
 
 // out[i] = sum over s of part[s * stride + i], s < n_parts (the fixed-order
-// second stage of every gradient and loss reduction): 32 outputs to a block, 32
-// threads to an output, thread k adding the parts k, k + 32, ...; the 32 sums are
-// added in order. One thread per output left a chain of up to 2,432 loads (190 us;
-// 8 now, for the head's 18 values).
-__global__ void __launch_bounds__(1024) reduce_parts_kernel(const float* __restrict__ part, int n_parts,
+// second stage of every gradient and loss reduction): 32 outputs to a block, K
+// threads to an output, thread k adding the parts k, k + K, ...; the K
+// sums are added in order. One thread per output left a chain of up to 2,432 loads
+// (190 us; 14 now, for the head's 18 values).
+template <int K>
+__global__ void __launch_bounds__(32 * K) reduce_parts_kernel(const float* __restrict__ part, int n_parts,
                                                             long long stride, int count, float* __restrict__ out) {
-    __shared__ float sum[32][33];
+    __shared__ float sum[K][33];
     const int i = blockIdx.x * 32 + threadIdx.x;
     float s = 0.0f;
     if (i < count) {
 #pragma unroll 4
-        for (int k = threadIdx.y; k < n_parts; k += 32) s += __ldg(part + (size_t)k * stride + i);
+        for (int k = threadIdx.y; k < n_parts; k += K) s += __ldg(part + (size_t)k * stride + i);
     }
     sum[threadIdx.y][threadIdx.x] = s;
     __syncthreads();
     if (threadIdx.y == 0 && i < count) {
         float t = 0.0f;
 #pragma unroll
-        for (int k = 0; k < 32; ++k) t += sum[k][threadIdx.x];
+        for (int k = 0; k < K; ++k) t += sum[k][threadIdx.x];
         out[i] = t;
     }
 }
 cudaError_t reduce_parts(const float* part, int n_parts, long long stride, int count, float* out, cudaStream_t st) {
-    reduce_parts_kernel<<<(count + 31) / 32, dim3(32, 32), 0, st>>>(part, n_parts, stride, count, out);
+    // 32 threads an output only for long chains: 19 parts of 442,000 outputs take 56
+    // us with 32 threads, 20 with 4
+    if (n_parts > 128) reduce_parts_kernel<32><<<(count + 31) / 32, dim3(32, 32), 0, st>>>(part, n_parts, stride, count, out);
+    else reduce_parts_kernel<8><<<(count + 31) / 32, dim3(32, 8), 0, st>>>(part, n_parts, stride, count, out);
     return cudaGetLastError();
 }
 
@@ -395,28 +543,6 @@ __global__ void pool_kernel(const __nv_bfloat16* __restrict__ x, __nv_bfloat16* 
 #pragma unroll
         for (int c = 0; c < 8; ++c) ob[c] = f2bf(0.125f * acc[c]);
         *reinterpret_cast<uint4*>(y + p * C + g * 8) = o;
-    }
-}
-
-// cat[v] = (low[parent(v)], skip[v]); fine side S, low has Cl channels, skip Cs.
-__global__ void upcat_kernel(const __nv_bfloat16* __restrict__ low, const __nv_bfloat16* __restrict__ skip,
-                             __nv_bfloat16* __restrict__ cat, int B, int S, int Cl, int Cs) {
-    const int C = Cl + Cs, g8 = C / 8, s = S / 2;
-    const long long total = (long long)B * S * S * S * g8;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total;
-         i += (long long)gridDim.x * blockDim.x) {
-        const int g = (int)(i % g8);
-        const long long v = i / g8;
-        const int x = (int)(v % S), y = (int)((v / S) % S), z = (int)((v / ((long long)S * S)) % S);
-        const long long bb = v / ((long long)S * S * S);
-        uint4 q;
-        if (g * 8 < Cl) {
-            const long long p = ((bb * s + z / 2) * s + y / 2) * s + x / 2;
-            q = *reinterpret_cast<const uint4*>(low + p * Cl + g * 8);
-        } else {
-            q = *reinterpret_cast<const uint4*>(skip + v * Cs + g * 8 - Cl);
-        }
-        *reinterpret_cast<uint4*>(cat + v * C + g * 8) = q;
     }
 }
 
@@ -479,112 +605,138 @@ __global__ void skip_back_kernel(const __nv_bfloat16* __restrict__ dpool, const 
 }
 
 // Weight gradient of a 3x3x3 layer, dW[tap][ci][co] = sum over samples and
-// voxels of x[v + tap - 1][ci] g[v][co], all 27 taps in one block: the block
-// stages a voxel tile of one sample (4 x 4 x 8 voxels: a 6 x 6 x 10 halo of x
-// and the tile of g, one 16-channel block of each, in FP32) once, and thread
-// (tap, ci) adds x[v + tap - 1][ci] g[v][0..15] for every voxel of the tile:
-// one x value and a broadcast row of g (every thread of the block reads the
-// same g row) per 16 FMAs. Thread (centre tap, ci 0) of the first ci block also
-// sums g for the bias gradient. Grid: x = voxel-tile split (split s takes the
-// tiles [s T / nsplit, (s + 1) T / nsplit)), y = ci block, z = co block; each
-// split writes its partial sums to its own slice of part ([split][27 cin cout +
-// cout]), which reduce_parts_kernel adds in split order.
+// voxels of x[v + tap - 1][ci] g[v][co], on the tensor cores: with K the voxels, A =
+// x^T (16 ci) seen through the tap's shift and B = g (NB co), both read from their
+// [voxel][channel] tiles by transposing matrix loads. tcgen05 takes M of 64 or 128
+// rows under one address, which 16 channels a tap do not make; mma.sync's 16 x 8 x
+// 16 fits them. A block stages voxel tiles (4 x 4 x 8: a 6 x 6 x 10 halo of x, the
+// first cl channels from low at half the resolution, and the tile of g; BF16, rows
+// padded so that 8 of them lie in distinct banks) through two buffers; warp (dz, dy)
+// holds the sums of its three taps. The products are exact; a tile's 128 are summed
+// in the tensor core from zero and the tiles' sums added in FP32, so that chains
+// are shorter than one FMA per voxel. Grid: x = tile split (split s takes the tiles
+// [s T / nsplit, (s + 1) T / nsplit)), y = ci block, z = co block; each split
+// writes its sums to its own slice of part ([split][27 cin cout + cout]). The FMAs
+// took 5.4 ms on 32 cubes of 32; this 0.7.
 constexpr int kDwD = 4, kDwH = 4, kDwW = 8, kDwVox = kDwD * kDwH * kDwW;
 constexpr int kDwHD = kDwD + 2, kDwHH = kDwH + 2, kDwHW = kDwW + 2, kDwHalo = kDwHD * kDwHH * kDwHW;
-constexpr int kDwThreads = 448;  // 27 taps x 16 ci = 432 accumulate; all stage
+constexpr int kDwThreads = 9 * 32;
+constexpr int kDwXRow = 48;  // bytes of a voxel's 16 channels and padding
+constexpr int dw_grow(int nb) { return 2 * nb + 16; }
+constexpr int dw_stage(int nb) { return kDwHalo * kDwXRow + kDwVox * dw_grow(nb); }
+constexpr int dw_nb(int cout) { return cout % 32 ? 16 : 32; }
 
+template <int NB>
 __global__ void __launch_bounds__(kDwThreads) dw_kernel(const __nv_bfloat16* __restrict__ x,
+                                                        const __nv_bfloat16* __restrict__ low, int cl,
                                                         const __nv_bfloat16* __restrict__ g,
                                                         float* __restrict__ part, int B, int S, int cin, int cout,
                                                         int nsplit) {
-    __shared__ float xs[kDwHalo][17];
-    __shared__ __align__(16) float gs[kDwVox][16];
+    extern __shared__ __align__(16) unsigned char dw_smem[];
+    constexpr int GROW = dw_grow(NB), NJ = NB / 8, P = kDwThreads / NB;
     const int cib = blockIdx.y, cob = blockIdx.z, split = blockIdx.x;
-    const int tid = threadIdx.x;
-    const int tap = tid >> 4, ci = tid & 15;
-    const bool acc_thread = tid < 27 * 16;
-    const bool bias_thread = cib == 0 && tap == 13 && ci == 0;
-    const int dz = tap / 9, dy = (tap / 3) % 3, dx = tap % 3;  // halo offsets of the tap
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int dz = warp / 3, dy = warp % 3;
     const int td = (S + kDwD - 1) / kDwD, th = (S + kDwH - 1) / kDwH, tw = (S + kDwW - 1) / kDwW;
     const long long T = (long long)B * td * th * tw;
     const long long t0 = T * split / nsplit, t1 = T * (split + 1) / nsplit;
-    float acc[16], bacc[16];
-#pragma unroll
-    for (int k = 0; k < 16; ++k) acc[k] = bacc[k] = 0.0f;
-    for (long long t = t0; t < t1; ++t) {
+    const bool lo = cib * 16 < cl;
+    const int sh = lo ? 1 : 0, Sx = S >> sh, ch = lo ? cl : cin - cl;
+    const __nv_bfloat16* xc = lo ? low + cib * 16 : x + cib * 16 - cl;
+    const auto stage = [&](long long t, int buf) {
         long long r = t;
-        const int iw = (int)(r % tw);
+        const int w0 = (int)(r % tw) * kDwW;
         r /= tw;
-        const int ih = (int)(r % th);
+        const int h0 = (int)(r % th) * kDwH;
         r /= th;
-        const int id = (int)(r % td);
+        const int d0 = (int)(r % td) * kDwD;
         const int b = (int)(r / td);
-        const int d0 = id * kDwD, h0 = ih * kDwH, w0 = iw * kDwW;
-        __syncthreads();  // the previous tile's values are no longer read
-        // stage: x halo (each item: 8 channels of one voxel) and the g tile
-        for (int u = tid; u < 2 * kDwHalo + 2 * kDwVox; u += kDwThreads) {
-            const bool isx = u < 2 * kDwHalo;
-            const int uu = isx ? u : u - 2 * kDwHalo;
-            const int half = uu & 1, vx = uu >> 1;
-            int d, h, w;
-            if (isx) {
-                d = d0 - 1 + vx / (kDwHH * kDwHW);
-                h = h0 - 1 + (vx / kDwHW) % kDwHH;
-                w = w0 - 1 + vx % kDwHW;
-            } else {
-                d = d0 + vx / (kDwH * kDwW);
-                h = h0 + (vx / kDwW) % kDwH;
-                w = w0 + vx % kDwW;
-            }
-            float v8[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-            if (d >= 0 && d < S && h >= 0 && h < S && w >= 0 && w < S) {
-                const long long vox = (((long long)b * S + d) * S + h) * S + w;
-                const uint4 q = isx ? *reinterpret_cast<const uint4*>(x + vox * cin + cib * 16 + half * 8)
-                                    : *reinterpret_cast<const uint4*>(g + vox * cout + cob * 16 + half * 8);
-                const __nv_bfloat16* qb = reinterpret_cast<const __nv_bfloat16*>(&q);
+        unsigned char* xs = dw_smem + buf * dw_stage(NB);
+        unsigned char* gs = xs + kDwHalo * kDwXRow;
+        for (int u = tid; u < 2 * kDwHalo; u += kDwThreads) {
+            const int half = u & 1, vx = u >> 1;
+            const int d = d0 - 1 + vx / (kDwHH * kDwHW), h = h0 - 1 + (vx / kDwHW) % kDwHH, w = w0 - 1 + vx % kDwHW;
+            const bool in = (unsigned)d < (unsigned)S && (unsigned)h < (unsigned)S && (unsigned)w < (unsigned)S;
+            const __nv_bfloat16* src =
+                in ? xc + ((((long long)b * Sx + (d >> sh)) * Sx + (h >> sh)) * Sx + (w >> sh)) * ch + half * 8 : x;
+            tc::cp_async16(xs + vx * kDwXRow + half * 16, src, in ? 16u : 0u);
+        }
+        for (int u = tid; u < kDwVox * NJ; u += kDwThreads) {
+            const int o = u % NJ, vx = u / NJ;
+            const int d = d0 + vx / (kDwH * kDwW), h = h0 + (vx / kDwW) % kDwH, w = w0 + vx % kDwW;
+            const bool in = d < S && h < S && w < S;
+            const __nv_bfloat16* src =
+                in ? g + ((((long long)b * S + d) * S + h) * S + w) * cout + cob * NB + o * 8 : g;
+            tc::cp_async16(gs + vx * GROW + o * 16, src, in ? 16u : 0u);
+        }
+        tc::cp_async_commit();
+    };
+    float sum[3][NJ][4], bsum = 0.0f;
 #pragma unroll
-                for (int e = 0; e < 8; ++e) v8[e] = bf2f(qb[e]);
-            }
-            float* dst = isx ? &xs[vx][half * 8] : &gs[vx][half * 8];
-#pragma unroll
-            for (int e = 0; e < 8; ++e) dst[e] = v8[e];
+    for (int i = 0; i < 3 * NJ * 4; ++i) (&sum[0][0][0])[i] = 0.0f;
+    // lane's row of the transposing loads: voxel w = lane & 7 of tile row 2 ks + hi
+    const int xrow = lane >> 4, xcol = ((lane >> 3) & 1) * 16;
+    const int grow = (lane >> 3) & 1, gcol = (lane >> 4) * 16;
+    const uint32_t base = tc::smem_addr(dw_smem);
+    if (t0 < t1) stage(t0, 0);
+    for (long long t = t0; t < t1; ++t) {
+        const int buf = (int)((t - t0) & 1);
+        if (t + 1 < t1) {
+            stage(t + 1, buf ^ 1);
+            tc::cp_async_wait<1>();
+        } else {
+            tc::cp_async_wait<0>();
         }
         __syncthreads();
-        if (acc_thread) {
-            // row by row of the tile: the tap's halo row, then 8 voxels along w
-            for (int vd = 0; vd < kDwD; ++vd)
-                for (int vh = 0; vh < kDwH; ++vh) {
-                    const float* xrow = &xs[((vd + dz) * kDwHH + (vh + dy)) * kDwHW + dx][ci];
-                    const float4* grow = reinterpret_cast<const float4*>(gs[(vd * kDwH + vh) * kDwW]);
+        const uint32_t xs = base + buf * dw_stage(NB), gs = xs + kDwHalo * kDwXRow;
+        float c[3][NJ][4];
 #pragma unroll
-                    for (int vw = 0; vw < kDwW; ++vw) {
-                        const float xv = xrow[vw * 17];
+        for (int i = 0; i < 3 * NJ * 4; ++i) (&c[0][0][0])[i] = 0.0f;
 #pragma unroll
-                        for (int q = 0; q < 4; ++q) {
-                            const float4 gq = grow[vw * 4 + q];
-                            acc[4 * q + 0] = fmaf(xv, gq.x, acc[4 * q + 0]);
-                            acc[4 * q + 1] = fmaf(xv, gq.y, acc[4 * q + 1]);
-                            acc[4 * q + 2] = fmaf(xv, gq.z, acc[4 * q + 2]);
-                            acc[4 * q + 3] = fmaf(xv, gq.w, acc[4 * q + 3]);
-                            if (bias_thread) {
-                                bacc[4 * q + 0] += gq.x;
-                                bacc[4 * q + 1] += gq.y;
-                                bacc[4 * q + 2] += gq.z;
-                                bacc[4 * q + 3] += gq.w;
-                            }
-                        }
-                    }
-                }
+        for (int ks = 0; ks < kDwVox / 16; ++ks) {
+            const int rx = 2 * ks + xrow, rg = 2 * ks + grow;
+            uint32_t bf[NJ / 2][4];
+#pragma unroll
+            for (int j = 0; j < NJ / 2; ++j)
+                tc::ldmatrix4_trans(gs + (rg * kDwW + (lane & 7)) * GROW + gcol + j * 32, bf[j]);
+#pragma unroll
+            for (int dx = 0; dx < 3; ++dx) {
+                uint32_t af[4];
+                tc::ldmatrix4_trans(
+                    xs + (((rx / kDwH + dz) * kDwHH + rx % kDwH + dy) * kDwHW + (lane & 7) + dx) * kDwXRow + xcol, af);
+#pragma unroll
+                for (int j = 0; j < NJ; ++j)
+                    tc::mma16816(c[dx][j], af, bf[j / 2][(j & 1) * 2], bf[j / 2][(j & 1) * 2 + 1]);
+            }
         }
+#pragma unroll
+        for (int i = 0; i < 3 * NJ * 4; ++i) (&sum[0][0][0])[i] += (&c[0][0][0])[i];
+        if (cib == 0 && tid < P * NB) {
+            const unsigned char* gp = dw_smem + buf * dw_stage(NB) + kDwHalo * kDwXRow + (tid % NB) * 2;
+            for (int vx = tid / NB; vx < kDwVox; vx += P)
+                bsum += bf2f(*reinterpret_cast<const __nv_bfloat16*>(gp + vx * GROW));
+        }
+        __syncthreads();  // the buffer is staged again
     }
-    if (acc_thread) {
-        float* dw = part + (size_t)split * ((size_t)27 * cin * cout + cout);
-        float* row = dw + ((size_t)tap * cin + cib * 16 + ci) * cout + cob * 16;
+    float* dw = part + (size_t)split * ((size_t)27 * cin * cout + cout);
 #pragma unroll
-        for (int k = 0; k < 16; ++k) row[k] = acc[k];
-        if (bias_thread) {
+    for (int dx = 0; dx < 3; ++dx)
 #pragma unroll
-            for (int k = 0; k < 16; ++k) dw[(size_t)27 * cin * cout + cob * 16 + k] = bacc[k];
+        for (int j = 0; j < NJ; ++j) {
+            float* row = dw + ((size_t)(warp * 3 + dx) * cin + cib * 16 + (lane >> 2)) * cout + cob * NB + j * 8 + (lane & 3) * 2;
+            row[0] = sum[dx][j][0];
+            row[1] = sum[dx][j][1];
+            row[(size_t)8 * cout] = sum[dx][j][2];
+            row[(size_t)8 * cout + 1] = sum[dx][j][3];
+        }
+    if (cib == 0) {
+        float* bs = reinterpret_cast<float*>(dw_smem);
+        bs[tid] = bsum;
+        __syncthreads();
+        if (tid < NB) {
+            float s = 0.0f;
+            for (int p = 0; p < P; ++p) s += bs[p * NB + tid];
+            dw[(size_t)27 * cin * cout + cob * NB + tid] = s;
         }
     }
 }
@@ -733,13 +885,16 @@ cudaError_t pack_weights(const float* w, __nv_bfloat16* wp, int cin, int cout, i
     return cudaGetLastError();
 }
 
-cudaError_t conv3_tc(const __nv_bfloat16* x, const __nv_bfloat16* wp, const float* bias, const __nv_bfloat16* mask,
-                     __nv_bfloat16* y, int B, int D, int H, int W, int cin, int cout, int epi, int* err, int n_sm,
-                     cudaStream_t st) {
-    (void)n_sm;
+// As conv3_tc of the header, with the first cl of the cin channels from low
+// (half the resolution, nearest up-sampling).
+static cudaError_t conv3_up(const __nv_bfloat16* x, const __nv_bfloat16* low, int cl, const __nv_bfloat16* wp,
+                            const float* bias, const __nv_bfloat16* mask, __nv_bfloat16* y, int B, int D, int H, int W,
+                            int cin, int cout, int epi, int* err, int n_sm, cudaStream_t st) {
     if (cin % 16 || cout % 16 || cout < 16 || cout > 256 || B < 1) return cudaErrorInvalidValue;
     ConvArgs a;
     a.x = x;
+    a.low = low;
+    a.cl = cl;
     a.wp = wp;
     a.bias = bias;
     a.mask = mask;
@@ -751,54 +906,68 @@ cudaError_t conv3_tc(const __nv_bfloat16* x, const __nv_bfloat16* wp, const floa
     a.cin = cin;
     a.cout = cout;
     a.epi = epi;
-    // Output depth per CTA: 4 D slices (fewer when the accumulators need more
-    // than 512 TMEM columns). Deeper tiles reuse the staged halo tile more but
-    // leave one CTA per SM whose 128 threads stage too slowly to keep the
-    // tensor cores fed (measured slower on GB300); double-buffered chunks when
-    // the input has more than one chunk and two stages fit.
-    // Folded layers: 8 (16 outputs) or 4 (32 outputs) slices per tile, the
-    // tile's DT + 4 accumulator slices (two of them on each side only collect
-    // halo contributions) in at most 256 TMEM columns.
+    a.err = err;
     a.fold = conv_folds(cout) ? 1 : 0;
-    int DT = a.fold ? (cout <= 16 ? 8 : 4) : 4;
-    while (!a.fold && DT > 1 && DT * cout > 512) --DT;
-    if (DT > D) DT = D;
-    const size_t stage_b = (size_t)2 * (DT + 2) * kHH * kWW * 16 + (size_t)27 * cout * 32;
-    const int nbuf = (2 * stage_b + 128 <= 200 * 1024 && cin > 16) ? 2 : 1;
-    if (DT < 1) return cudaErrorInvalidValue;
-    a.DT = DT;
-    int nc = 32;
-    while (nc < (DT + (a.fold ? 4 : 0)) * cout) nc *= 2;
-    a.ncols = nc;
-    a.itile = (uint32_t)(DT + 2) * kHH * kWW * 16;
-    a.wtile = 27u * (uint32_t)cout * 32u;
-    a.stage = 2 * a.itile + a.wtile;
-    a.nbuf = nbuf;
+    // At most 64 output channels a tile: two stages with 27 taps of weights fit,
+    // and the deepest level has tiles for all SMs.
+    a.nsplit = 1;
+    while (cout / a.nsplit > 64 || cout % (16 * a.nsplit)) ++a.nsplit;
+    a.nb = cout / a.nsplit;
+    a.wtile = 27u * (uint32_t)a.nb * 32u;
     a.tiles_w = (W + kTW - 1) / kTW;
     a.tiles_h = (H + kTH - 1) / kTH;
-    a.tiles_d = (D + DT - 1) / DT;
-    a.err = err;
-    size_t smem = (size_t)a.nbuf * a.stage + 128;
-    // keep (CTAs per SM) x (TMEM columns) within the 512 columns of an SM
-    const size_t sm_bytes = 228 * 1024, per_cta_reserve = 1024 + 64;
-    const int max_ctas = 512 / nc;
-    if ((sm_bytes / (smem + per_cta_reserve)) > (size_t)max_ctas) smem = sm_bytes / max_ctas - per_cta_reserve + 1;
-    if (smem > 227 * 1024) return cudaErrorInvalidValue;
+    const size_t room = 227 * 1024 - 4096;
+    const int nch = cin / 16;
+    a.resident = a.nsplit == 1 && (size_t)nch * a.wtile <= 64 * 1024;
+    // Depth of the tiles: the deeper, the less halo per output; the shallower, the
+    // evener the SMs' shares. The cost (clocks) of a chunk is its MMAs' (an operand
+    // read of 4 KB or N / 2 columns each) or its staging's, whichever is longer.
+    const int most = a.fold ? (cout <= 16 ? 8 : 4) : 4;
+    double best = 0.0;
+    long long tiles = 0;
+    for (int DT = 1; DT <= most && DT <= D; ++DT) {
+        const long long n = (long long)a.tiles_w * a.tiles_h * ((D + DT - 1) / DT) * B * a.nsplit;
+        const double mma = (a.fold ? 9.0 * (DT + 2) : 27.0 * DT) * std::max(40.0, 0.55 * a.nb * (a.fold ? 3 : 1));
+        const double load = 110.0 * (DT + 2) + (a.resident ? 0.0 : a.wtile / 64.0);
+        const double cost = (double)((n + n_sm - 1) / n_sm) * (nch * std::max(mma, load) + 1000.0);
+        if (DT == 1 || cost < best) {
+            best = cost;
+            a.DT = DT;
+            tiles = n;
+        }
+    }
+    if (tiles > 0x7fffffffLL || (long long)D * H * W * cin > 0x7fffffffLL) return cudaErrorInvalidValue;
+    a.n_tiles = (int)tiles;
+    a.tiles_d = (D + a.DT - 1) / a.DT;
+    a.acc_cols = (a.DT + (a.fold ? 4 : 0)) * a.nb;
+    a.n_acc = 2 * a.acc_cols <= 512 ? 2 : 1;
+    a.ncols = 32;
+    while (a.ncols < a.n_acc * a.acc_cols) a.ncols *= 2;
+    a.itile = (uint32_t)(a.DT + 2) * kHH * kWW * 16;
+    a.stage = 2 * a.itile + (a.resident ? 0u : a.wtile);
+    const size_t fixed = a.resident ? (size_t)nch * a.wtile : 0;
+    a.n_stage = (int)std::min<size_t>(kStages, (room - fixed) / a.stage);
+    if (a.n_stage < 1 || a.ncols > 512) return cudaErrorInvalidValue;
+    const size_t smem = fixed + (size_t)a.n_stage * a.stage + 128;
     UCK(cudaFuncSetAttribute(conv3_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    const long long nblk = (long long)a.tiles_w * a.tiles_h * a.tiles_d * B;
-    if (nblk > 0x7fffffffLL) return cudaErrorInvalidValue;
-    conv3_tc_kernel<<<(unsigned)nblk, 128, smem, st>>>(a);
+    conv3_tc_kernel<<<std::min(a.n_tiles, n_sm), kConvThreads, smem, st>>>(a);
     return cudaGetLastError();
+}
+
+cudaError_t conv3_tc(const __nv_bfloat16* x, const __nv_bfloat16* wp, const float* bias, const __nv_bfloat16* mask,
+                     __nv_bfloat16* y, int B, int D, int H, int W, int cin, int cout, int epi, int* err, int n_sm,
+                     cudaStream_t st) {
+    return conv3_up(x, nullptr, 0, wp, bias, mask, y, B, D, H, W, cin, cout, epi, err, n_sm, st);
 }
 
 // ---- network driver --------------------------------------------------------
 
-// Voxel-tile splits of a weight-gradient launch: about eight blocks per SM
-// over the (ci, co) blocks, and no split without a tile.
+// Voxel-tile splits of a weight-gradient launch: about four blocks per SM over
+// the (ci, co) blocks, and no split without a tile.
 static int dw_splits(int B, int S, int cin, int cout, int n_sm) {
     const long long tiles = (long long)B * ((S + kDwD - 1) / kDwD) * ((S + kDwH - 1) / kDwH) * ((S + kDwW - 1) / kDwW);
-    const long long cb = (long long)(cin / 16) * (cout / 16);
-    const long long want = std::max(1LL, 8LL * n_sm / cb);
+    const long long cb = (long long)(cin / 16) * (cout / dw_nb(cout));
+    const long long want = std::max(1LL, 4LL * n_sm / cb);
     return (int)std::max(1LL, std::min(tiles, want));
 }
 
@@ -839,13 +1008,10 @@ cudaError_t create(Net& n, int S, int Bmax) {
     UCK(act(&n.p2, v3, 64));
     UCK(act(&n.x3a, v3, 128));
     UCK(act(&n.x3, v3, 128));
-    UCK(act(&n.c2, v2, 192));
     UCK(act(&n.y2a, v2, 64));
     UCK(act(&n.y2, v2, 64));
-    UCK(act(&n.c1, v1, 96));
     UCK(act(&n.y1a, v1, 32));
     UCK(act(&n.y1, v1, 32));
-    UCK(act(&n.c0, v0, 48));
     UCK(act(&n.y0a, v0, 16));
     UCK(act(&n.y0, v0, 16));
     UCK(act(&n.g_y0, v0, 16));
@@ -908,11 +1074,13 @@ cudaError_t forward(Net& n, const float* in, int B, cudaStream_t st) {
     if (!n.packed) UCK(pack(n, st));
     const int S = n.S, S1 = S / 2, S2 = S / 4, S3 = S / 8;
     const long long v0 = (long long)B * S * S * S, v1 = v0 / 8, v2 = v1 / 8, v3 = v2 / 8;
-    auto conv = [&](const __nv_bfloat16* x, __nv_bfloat16* y, int l, int s) {
-        return conv3_tc(x, n.wfwd[l], bias_of(n, l), nullptr, y, B, s, s, s, kCin[l], kCout[l], 1, n.d_err, n.n_sm,
-                        st);
+    auto conv_up = [&](const __nv_bfloat16* x, const __nv_bfloat16* low, int cl, __nv_bfloat16* y, int l, int s) {
+        return conv3_up(x, low, cl, n.wfwd[l], bias_of(n, l), nullptr, y, B, s, s, s, kCin[l], kCout[l], 1, n.d_err,
+                        n.n_sm, st);
     };
-    conv_first_kernel<<<grid_for(v0, n.n_sm), 256, 0, st>>>(in, n.params, bias_of(n, 0), n.x0a, B, S);
+    auto conv = [&](const __nv_bfloat16* x, __nv_bfloat16* y, int l, int s) { return conv_up(x, nullptr, 0, y, l, s); };
+    const auto first = reinterpret_cast<uintptr_t>(in) % 16 ? conv_first_kernel<false> : conv_first_kernel<true>;
+    first<<<grid_for(v0 / 4, n.n_sm), 256, 0, st>>>(in, n.params, bias_of(n, 0), n.x0a, B, S);
     UCK(cudaGetLastError());
     UCK(conv(n.x0a, n.x0, 1, S));
     pool_kernel<<<grid_for(v1 * 2, n.n_sm), 256, 0, st>>>(n.x0, n.p0, B, S, 16);
@@ -924,14 +1092,11 @@ cudaError_t forward(Net& n, const float* in, int B, cudaStream_t st) {
     pool_kernel<<<grid_for(v3 * 8, n.n_sm), 256, 0, st>>>(n.x2, n.p2, B, S2, 64);
     UCK(conv(n.p2, n.x3a, 6, S3));
     UCK(conv(n.x3a, n.x3, 7, S3));
-    upcat_kernel<<<grid_for(v2 * 24, n.n_sm), 256, 0, st>>>(n.x3, n.x2, n.c2, B, S2, 128, 64);
-    UCK(conv(n.c2, n.y2a, 8, S2));
+    UCK(conv_up(n.x2, n.x3, 128, n.y2a, 8, S2));
     UCK(conv(n.y2a, n.y2, 9, S2));
-    upcat_kernel<<<grid_for(v1 * 12, n.n_sm), 256, 0, st>>>(n.y2, n.x1, n.c1, B, S1, 64, 32);
-    UCK(conv(n.c1, n.y1a, 10, S1));
+    UCK(conv_up(n.x1, n.y2, 64, n.y1a, 10, S1));
     UCK(conv(n.y1a, n.y1, 11, S1));
-    upcat_kernel<<<grid_for(v0 * 6, n.n_sm), 256, 0, st>>>(n.y1, n.x0, n.c0, B, S, 32, 16);
-    UCK(conv(n.c0, n.y0a, 12, S));
+    UCK(conv_up(n.x0, n.y1, 32, n.y0a, 12, S));
     UCK(conv(n.y0a, n.y0, 13, S));
     head_kernel<<<grid_for(v0, n.n_sm), 256, 0, st>>>(n.y0, n.params + param_offset(kHead), n.out, v0);
     return cudaGetLastError();
@@ -956,30 +1121,36 @@ cudaError_t backward(Net& n, const float* in, const float* target, int B, cudaSt
         return conv3_tc(g, n.wbwd[l], nullptr, xmask, dx, B, s, s, s, kCout[l], kCin[l], xmask ? 2 : 0, n.d_err,
                         n.n_sm, st);
     };
-    auto dweight = [&](const __nv_bfloat16* x, const __nv_bfloat16* g, int l, int s) {
+    auto dweight_up = [&](const __nv_bfloat16* x, const __nv_bfloat16* low, int cl, const __nv_bfloat16* g, int l, int s) {
         const int nsplit = dw_splits(B, s, kCin[l], kCout[l], n.n_sm);
-        dim3 grid(nsplit, kCin[l] / 16, kCout[l] / 16);
+        const int nb = dw_nb(kCout[l]), smem = 2 * dw_stage(nb);
+        const auto f = nb == 16 ? dw_kernel<16> : dw_kernel<32>;
+        UCK(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+        dim3 grid(nsplit, kCin[l] / 16, kCout[l] / nb);
         const int count = 27 * kCin[l] * kCout[l] + kCout[l];
-        dw_kernel<<<grid, kDwThreads, 0, st>>>(x, g, n.gpart, B, s, kCin[l], kCout[l], nsplit);
+        f<<<grid, kDwThreads, smem, st>>>(x, low, cl, g, n.gpart, B, s, kCin[l], kCout[l], nsplit);
         UCK(cudaGetLastError());
         return reduce_parts(n.gpart, nsplit, count, count, n.grads + param_offset(l), st);
+    };
+    auto dweight = [&](const __nv_bfloat16* x, const __nv_bfloat16* g, int l, int s) {
+        return dweight_up(x, nullptr, 0, g, l, s);
     };
     // level 0, up path
     UCK(dweight(n.y0a, n.g_y0, 13, S));
     UCK(dconv(n.g_y0, n.y0a, n.g_y0a, 13, S));
-    UCK(dweight(n.c0, n.g_y0a, 12, S));
+    UCK(dweight_up(n.x0, n.y1, 32, n.g_y0a, 12, S));
     UCK(dconv(n.g_y0a, nullptr, n.g_c0, 12, S));
     upcat_back_low_kernel<<<grid_for(v1 * 4, n.n_sm), 256, 0, st>>>(n.g_c0, n.y1, n.g_y1, B, S, 32, 16);
     // level 1, up path
     UCK(dweight(n.y1a, n.g_y1, 11, S1));
     UCK(dconv(n.g_y1, n.y1a, n.g_y1a, 11, S1));
-    UCK(dweight(n.c1, n.g_y1a, 10, S1));
+    UCK(dweight_up(n.x1, n.y2, 64, n.g_y1a, 10, S1));
     UCK(dconv(n.g_y1a, nullptr, n.g_c1, 10, S1));
     upcat_back_low_kernel<<<grid_for(v2 * 8, n.n_sm), 256, 0, st>>>(n.g_c1, n.y2, n.g_y2, B, S1, 64, 32);
     // level 2, up path
     UCK(dweight(n.y2a, n.g_y2, 9, S2));
     UCK(dconv(n.g_y2, n.y2a, n.g_y2a, 9, S2));
-    UCK(dweight(n.c2, n.g_y2a, 8, S2));
+    UCK(dweight_up(n.x2, n.x3, 128, n.g_y2a, 8, S2));
     UCK(dconv(n.g_y2a, nullptr, n.g_c2, 8, S2));
     upcat_back_low_kernel<<<grid_for(v3 * 16, n.n_sm), 256, 0, st>>>(n.g_c2, n.x3, n.g_x3, B, S2, 128, 64);
     // bottleneck

@@ -45,7 +45,7 @@ struct Net {
     // activations (BF16, channels last) and their gradients, sized for Bmax
     std::vector<void*> bufs;
     __nv_bfloat16 *x0a, *x0, *p0, *x1a, *x1, *p1, *x2a, *x2, *p2, *x3a, *x3;
-    __nv_bfloat16 *c2, *y2a, *y2, *c1, *y1a, *y1, *c0, *y0a, *y0;
+    __nv_bfloat16 *y2a, *y2, *y1a, *y1, *y0a, *y0;
     __nv_bfloat16 *g_y0, *g_y0a, *g_c0, *g_y1, *g_y1a, *g_c1, *g_y2, *g_y2a, *g_c2;
     __nv_bfloat16 *g_x3, *g_x3a, *g_p2, *g_x2, *g_x2a, *g_p1, *g_x1, *g_x1a, *g_p0, *g_x0, *g_x0a;
     float* out = nullptr;           // [Bmax][S^3] FP32 network output
