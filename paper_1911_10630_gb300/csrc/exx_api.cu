@@ -23,7 +23,7 @@ cudaError_t launch_pair_list(int n, const double* centers, const double L[3], co
                              PairRec* pairs, cudaStream_t st, const double* alphas, double ln_inv_eps,
                              double delta_max, int r_min, int ns_pe = 0, int ns_me = 0, int* bad = nullptr);
 cudaError_t launch_radii_sort(const PairRec* pairs, const int* n_pair, int* hist, int n_geo, int* order, int num_sms,
-                              cudaStream_t st, int* classes = nullptr);
+                              cudaStream_t st, int* classes = nullptr, const int* rank = nullptr);
 cudaError_t cluster_set_smem(int variant, size_t smem);
 cudaError_t launch_zero(double* p, long long n, int num_sms, cudaStream_t st);
 cudaError_t launch_box_clip(const PairRec* pairs, const int* n_pair, const int* box_org, const int bdim[3],
@@ -141,7 +141,8 @@ struct exx_ctx {
     // side by side on the context stream and the aux streams; each launch has
     // its own workspace slots
     struct MarchClass {
-        int threads = 0, g_lo = 0, g_hi = 0, slots = 0;
+        int threads = 0, r_lo = 0, r_hi = 0, slots = 0;  // ranks of its balls in the order
+        bool general = false;     // balls that stay on pair_kernel
         size_t smem = 0, at = 0, hot = 0;  // dynamic shared memory; first bytes of its slots
         SolveParams P;            // slot offsets and sizes of the class (the rest as in the context's P)
     };
@@ -149,6 +150,9 @@ struct exx_ctx {
     char* march_ws = nullptr;
     void* march_mem = nullptr;   // device tables
     int2* d_march_range = nullptr;
+    int* d_march_rank = nullptr; // [n_geo] place of a ball in the order (several classes)
+    bool march_general = false;  // one of the classes is pair_kernel's
+    int pk_threads = 0;          // pair_kernel's threads
     int* d_march_cls = nullptr;  // [2 classes] start and length in the order, [classes] work counters
     cudaStream_t march_st[5] = {};
     cudaEvent_t march_ev[6] = {};  // joins of the aux streams, [5] fork
@@ -483,30 +487,59 @@ static cudaError_t launch_cg64(exx_ctx* c, const SolveParams& P, int n, cudaStre
 // CTA size of the marching multigrid CG for a ball of n columns: one each.
 static int march_threads(int n) { return n <= 128 ? 128 : (n <= 256 ? 256 : 512); }
 
+// Whether a ball's multigrid PCG holds in FP32: at most one of its coarse balls
+// reaches beyond its fine one (2 R_{l+1} > R_l). Where two do, the PCG carries
+// rounding errors of 1e-7 up a hundredfold, so that every order of its sums stops
+// somewhere else within the tolerance: at tol 1e-8, D_xx on another CTA size differs
+// by 7e-10 to 1.2e-9 (R_PE 17, 21, 25, 34), against 1e-11 (16, 24, 32). Those balls
+// stay on pair_kernel, whose results callers have.
+static bool march_steady(int R) {
+    int over = 0;
+    for (; R > 3; R = (R + 1) / 2) over += R & 1;
+    return over <= 1;
+}
+
 // Plans the marching multigrid CG: classes of radii by CTA size, tables and
 // slot layouts. Leaves c->march empty when a ball has no coarse level or is
-// larger than the largest CTA holds, or when the requested threads do not hold
-// the largest ball's columns (pair_kernel then runs the call).
+// larger than the largest CTA holds, when the requested threads do not hold
+// the largest ball's columns, or when no ball is steady (pair_kernel then runs
+// the call).
 static exx_status plan_march(exx_ctx* c, const std::vector<std::vector<HostMGLevel>>& mgl) {
     const int ng = c->n_geo, want = c->opt.threads;
     const bool asked = want == 256 || want == 512 || want == 1024;
     std::vector<HostMarch> H(ng);
-    std::vector<int> nt(ng);
+    std::vector<int> nt(ng, 0);  // 0: pair_kernel
     const int largest = march_threads(march_columns(c->balls[ng - 1].r_pe));
+    bool any = false;
     for (int g = 0; g < ng; ++g) {
-        nt[g] = asked ? want : march_threads(march_columns(c->balls[g].r_pe));
+        const int R = c->balls[g].r_pe;
+        if (R > 35 || R <= 3) return EXX_OK;
+        if (!march_steady(R)) {
+            c->march_general = true;
+            H[g].G = MarchGeo();
+            continue;
+        }
+        nt[g] = asked ? want : march_threads(march_columns(R));
         if (!asked && nt[g] == largest) nt[g] = std::max(nt[g], 256);  // the largest ball's class
-        if (c->balls[g].r_pe > 35 || !build_march(c->balls[g], mgl[g], nt[g], H[g])) return EXX_OK;
+        if (!build_march(c->balls[g], mgl[g], nt[g], H[g])) {
+            c->march_general = false;
+            return EXX_OK;
+        }
+        any = true;
+    }
+    if (!any) {
+        c->march_general = false;
+        return EXX_OK;
     }
     // tables
-    size_t bytes = align256(sizeof(MarchGeo) * ng) + align256(sizeof(int2) * ng);
+    size_t bytes = align256(sizeof(MarchGeo) * ng) + align256(sizeof(int2) * ng) + align256(sizeof(int) * ng);
     for (const HostMarch& h : H) {
         for (const HostMarchLv& l : h.lv) bytes += align256(sizeof(int) * l.col.size()) + align256(sizeof(int) * l.pst.size());
         bytes += align256(sizeof(int) * h.qidx.size());
     }
     CK(cudaMalloc(&c->march_mem, bytes), "cudaMalloc(marching tables)");
     std::vector<char> host(bytes, 0);
-    size_t at = align256(sizeof(MarchGeo) * ng) + align256(sizeof(int2) * ng);
+    size_t at = align256(sizeof(MarchGeo) * ng) + align256(sizeof(int2) * ng) + align256(sizeof(int) * ng);
     auto put = [&](const std::vector<int>& v) -> char* {
         std::memcpy(host.data() + at, v.data(), sizeof(int) * v.size());
         char* p = (char*)c->march_mem + at;
@@ -520,15 +553,30 @@ static exx_status plan_march(exx_ctx* c, const std::vector<std::vector<HostMGLev
         }
         h.G.qidx = (const int*)put(h.qidx);
     }
-    // classes, the largest balls first
-    for (int g = ng - 1; g >= 0;) {
+    // classes, the largest CTAs first and pair_kernel's last; ranks ascend within
+    // and across them in the opposite order
+    std::vector<int> rank(ng), sizes(nt);
+    std::sort(sizes.begin(), sizes.end());
+    sizes.erase(std::unique(sizes.begin(), sizes.end()), sizes.end());
+    int next = 0;
+    for (int size : sizes) {
         exx_ctx::MarchClass K;
-        K.threads = nt[g];
-        K.g_hi = g;
-        while (g >= 0 && nt[g] == K.threads) --g;
-        K.g_lo = g + 1;
+        K.threads = size;
+        K.r_lo = next;
+        std::vector<int> mine;
+        for (int g = 0; g < ng; ++g)
+            if (nt[g] == size) {
+                mine.push_back(g);
+                rank[g] = next++;
+            }
+        K.r_hi = next - 1;
         std::memset(&K.P, 0, sizeof(K.P));
-        const HostBall& B = c->balls[K.g_hi];
+        if (size == 0) {
+            K.general = true;
+            c->march.push_back(K);
+            continue;
+        }
+        const HostBall& B = c->balls[mine.back()];
         const size_t S3 = (size_t)(2 * c->r_me + 1) * (2 * c->r_me + 1) * (2 * c->r_me + 1);
         size_t off = 0;
         auto take = [&](size_t n) {
@@ -547,7 +595,7 @@ static exx_status plan_march(exx_ctx* c, const std::vector<std::vector<HostMGLev
         const size_t vec = 2 * sizeof(float4) * (size_t)march_row(K.threads);
         take(vec * kMarchVectors);
         size_t floats = 0;
-        for (int q = K.g_lo; q <= K.g_hi; ++q) {
+        for (int q : mine) {
             MarchGeo& M = H[q].G;
             floats = std::max(floats, (size_t)M.smem_floats);
             for (int l = 1; l < M.nm; ++l) {  // of its own for every ball: zero off the ball for good
@@ -559,21 +607,25 @@ static exx_status plan_march(exx_ctx* c, const std::vector<std::vector<HostMGLev
         K.smem = std::max(sizeof(float) * floats, sizeof(double) * (size_t)(2 * B.r_pe + 1) * 28);
         c->march.push_back(K);
     }
-    if (c->march.size() > 6) return fail(c, EXX_EINVAL, "exx_init: too many marching classes");
+    std::reverse(c->march.begin(), c->march.end());
     std::vector<MarchGeo> mg;
     for (HostMarch& h : H) mg.push_back(h.G);
     std::memcpy(host.data(), mg.data(), sizeof(MarchGeo) * ng);
     std::vector<int2> range;
-    for (const auto& K : c->march) range.push_back(make_int2(K.g_lo, K.g_hi));
+    for (const auto& K : c->march) range.push_back(make_int2(K.r_lo, K.r_hi));
     std::memcpy(host.data() + align256(sizeof(MarchGeo) * ng), range.data(), sizeof(int2) * range.size());
+    const size_t at_rank = align256(sizeof(MarchGeo) * ng) + align256(sizeof(int2) * ng);
+    std::memcpy(host.data() + at_rank, rank.data(), sizeof(int) * ng);
     CK(cudaMemcpy(c->march_mem, host.data(), bytes, cudaMemcpyHostToDevice), "cudaMemcpy(marching tables)");
     c->P.march = (const MarchGeo*)c->march_mem;
     c->d_march_range = (int2*)((char*)c->march_mem + align256(sizeof(MarchGeo) * ng));
+    c->d_march_rank = (int*)((char*)c->march_mem + at_rank);
     // slots: every CTA that can be resident, within a quarter of the free memory
     size_t free_b = 0, total_b = 0, need = 0;
     cudaMemGetInfo(&free_b, &total_b);
     for (auto& K : c->march) {
         int bps = 0;
+        if (K.general) continue;
         CK(march_occupancy(K.threads, K.smem, &bps), "occupancy query (marching kernel)");
         if (bps < 1) return fail(c, EXX_ECUDA, "marching kernel does not fit on an SM");
         K.slots = c->num_sms * (c->opt.ctas_per_sm > 0 ? std::min(c->opt.ctas_per_sm, bps) : bps);
@@ -581,7 +633,7 @@ static exx_status plan_march(exx_ctx* c, const std::vector<std::vector<HostMGLev
     }
     if (need > free_b / 4) {
         const double f = 0.25 * (double)free_b / (double)need;
-        for (auto& K : c->march) K.slots = std::max(1, (int)(K.slots * f));
+        for (auto& K : c->march) K.slots = K.general ? 0 : std::max(1, (int)(K.slots * f));
     }
     at = 0;
     for (auto& K : c->march) {
@@ -1193,8 +1245,9 @@ extern "C" exx_status exx_init(exx_ctx** out, const double cell[3], const int gr
     cudaMemGetInfo(&free_b, &total_b);
     long long fit = (long long)(0.25 * (double)free_b / (double)c->slot_bytes);
     c->n_slots = (int)std::max(1LL, std::min(want, fit));
-    if (!c->march.empty()) {  // pair_kernel's slots serve single-pair and operator queries only
-        c->n_slots = 1;
+    c->pk_threads = c->threads;
+    if (!c->march.empty()) {
+        if (!c->march_general) c->n_slots = 1;  // for single-pair and operator queries only
         c->threads = c->march[0].threads;
     }
     if (c->per_class && c->n_slots < want) {  // not enough memory for two lanes: one lane, shared slots
@@ -1291,6 +1344,7 @@ extern "C" exx_status exx_init(exx_ctx** out, const double cell[3], const int gr
     P.inner_max_iter = o.inner_max_iter;
     P.inner_tol = o.inner_tol;
     P.max_refine = 40;
+    P.few = o.precision == 1 && o.preconditioner == 1 ? 2 * c->num_sms : 0;
     P.update_drop = o.update_drop;
     P.lmax = l_max;
     P.n_mono = (l_max + 1) * (l_max + 2) * (l_max + 3) / 6;
@@ -1309,7 +1363,7 @@ extern "C" exx_status exx_init(exx_ctx** out, const double cell[3], const int gr
     c->stats.lane_map = c->use_cluster ? c->cands[c->cand].lane_map : 0;
     if (!c->march.empty()) {
         c->stats.grid_ctas = 0;
-        for (const auto& K : c->march) c->stats.grid_ctas += K.slots;
+        for (const auto& K : c->march) c->stats.grid_ctas += K.general ? c->n_slots : K.slots;
     }
     c->stats.n_candidates = (int)c->cands.size();
     c->stats.threads = c->threads;
@@ -1366,7 +1420,7 @@ static exx_status enqueue(exx_ctx* c, const double* orbitals, const double* cent
        "pair list");
     if (c->n_geo > 1)
         CK(launch_radii_sort(c->d_pairs, c->d_scalars, c->d_hist, c->n_geo, c->d_order, c->num_sms, st,
-                             c->per_class ? c->d_class : nullptr),
+                             c->per_class ? c->d_class : nullptr, c->march.size() > 1 ? c->d_march_rank : nullptr),
            "largest-first order");
     if (c->march.size() > 1)
         CK(launch_class_runs(c->d_hist, c->n_geo, c->d_march_range, (int)c->march.size(), c->d_march_cls, st),
@@ -1400,7 +1454,7 @@ static exx_status enqueue(exx_ctx* c, const double* orbitals, const double* cent
                                          RC.cand.smem, ls),
                    "cluster pair kernel (radius class)");
             else
-                CK(launch_pair_kernel(Pg, c->threads, true, slots, c->smem, ls), "pair kernel (radius class)");
+                CK(launch_pair_kernel(Pg, c->pk_threads, true, slots, c->smem, ls), "pair kernel (radius class)");
         }
         if (two) {
             CK(cudaEventRecord(c->ev_join, c->aux), "cudaEventRecord(join)");
@@ -1420,6 +1474,17 @@ static exx_status enqueue(exx_ctx* c, const double* orbitals, const double* cent
             cudaStream_t ks = k ? c->march_st[k - 1] : st;
             if (k) CK(cudaStreamWaitEvent(ks, c->march_ev[5], 0), "cudaStreamWaitEvent(fork)");
             SolveParams Pk = P;
+            if (nk > 1) {
+                Pk.item_base = c->d_march_cls + 2 * k;
+                Pk.n_pair = c->d_march_cls + 2 * k + 1;
+                Pk.queue = c->d_march_cls + 2 * nk + k;
+            }
+            if (K.general) {
+                CK(launch_pair_kernel(Pk, c->pk_threads, true, c->n_slots, c->smem, ks), "pair kernel");
+                CK(cudaEventRecord(c->march_ev[k - 1], ks), "cudaEventRecord(join)");
+                CK(cudaStreamWaitEvent(st, c->march_ev[k - 1], 0), "cudaStreamWaitEvent(join)");
+                continue;
+            }
             Pk.ws = c->march_ws + K.at;
             Pk.slot_bytes = K.P.slot_bytes;
             Pk.ws_hot = c->march_ws + K.hot;
@@ -1430,11 +1495,6 @@ static exx_status enqueue(exx_ctx* c, const double* orbitals, const double* cent
             Pk.off_sy = K.P.off_sy;
             Pk.off_ush = K.P.off_ush;
             Pk.off_rows = K.P.off_rows;
-            if (nk > 1) {
-                Pk.item_base = c->d_march_cls + 2 * k;
-                Pk.n_pair = c->d_march_cls + 2 * k + 1;
-                Pk.queue = c->d_march_cls + 2 * nk + k;
-            }
             CK(launch_march_kernel(Pk, K.threads, (int)std::min<long long>(K.slots, (long long)n * (n + 1) / 2), K.smem, ks),
                "marching pair kernel");
             if (k) {
@@ -1444,7 +1504,7 @@ static exx_status enqueue(exx_ctx* c, const double* orbitals, const double* cent
         }
     } else
         CK(c->cg64_ctas ? launch_cg64(c, P, n, st)
-                        : launch_pair_kernel(P, c->threads, c->opt.precision == 1, c->n_slots, c->smem, st),
+                        : launch_pair_kernel(P, c->pk_threads, c->opt.precision == 1, c->n_slots, c->smem, st),
            "pair kernel");
     if (P.dfix != 0.0)
         CK(launch_dfix_convert(d_xx, (long long)n * c->cur_ostride, 1.0 / P.dfix, c->num_sms, st), "D_xx to FP64");
@@ -2101,7 +2161,7 @@ extern "C" exx_status exx_debug_pair(exx_ctx* c, const double* orbitals, int ind
     exx_status s = EXX_OK;
     cudaError_t e = c->use_cluster ? launch_cluster_kernel(c->cl_variant, P, c->CL, 1, c->smem, st)
                     : c->cg64_ctas ? launch_cg64(c, P, 1, st)
-                                   : launch_pair_kernel(P, c->threads, c->opt.precision == 1, 1, c->smem, st);
+                                   : launch_pair_kernel(P, c->pk_threads, c->opt.precision == 1, 1, c->smem, st);
     if (e == cudaSuccess) e = launch_debug_readback(P, pr, d_rho, d_v, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (e == cudaSuccess && rho) e = cudaMemcpy(rho, d_rho, sizeof(double) * B.n_me, cudaMemcpyDeviceToHost);

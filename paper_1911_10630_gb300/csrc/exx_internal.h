@@ -201,6 +201,7 @@ struct SolveParams {
     int inner_max_iter;
     double inner_tol;
     int max_refine;
+    int few;              // pair_kernel, FP32 multigrid CG, 256 threads: up to so many pairs take 512 threads each (0: none)
     double update_drop;       // reliable-update trigger of the cluster solver
     unsigned long long* phase_clk;  // [4] cycles: setup, FP64 residuals, FP32 CG, finish (cluster solver)
     int lmax;

@@ -4,7 +4,7 @@
 // One persistent CTA per pair, the CTA sized to the ball: NT threads hold one
 // column each, 128 registers a thread, so an SM holds 512 threads (a multiple
 // of 128 a CTA: tensor memory ties a warp to a quarter of the SM). Per-pair
-// radii run as one launch per CTA size over the largest-first order.
+// radii run as one launch per CTA size, each over its run of the order.
 //
 // The FP64 phases around the PCG are bound by the FP64 pipe (two lanes a clock
 // and SM) and by latency at 16 warps an SM, so they spend few FP64 operations

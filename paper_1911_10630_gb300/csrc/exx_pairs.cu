@@ -193,12 +193,13 @@ __global__ void pairs_fill_kernel(int n, const double* __restrict__ C, PairGeom 
 }
 
 // Largest pairs first: counting sort of the pair indices by geometry
-// (descending radius). hist[0..n_geo) counts, hist[n_geo..2 n_geo) cursors.
+// (descending radius; or descending rank[geometry]). hist[0..n_geo) counts,
+// hist[n_geo..2 n_geo) cursors.
 __global__ void radii_count_kernel(const PairRec* __restrict__ pairs, const int* __restrict__ n_pair,
-                                   int* __restrict__ hist, int n_geo) {
+                                   const int* __restrict__ rank, int* __restrict__ hist, int n_geo) {
     const int np = *n_pair;
     for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < np; p += gridDim.x * blockDim.x)
-        atomicAdd(hist + pairs[p].geo, 1);
+        atomicAdd(hist + (rank ? rank[pairs[p].geo] : pairs[p].geo), 1);
 }
 
 __global__ void radii_scan_kernel(int* __restrict__ hist, int n_geo) {
@@ -212,10 +213,10 @@ __global__ void radii_scan_kernel(int* __restrict__ hist, int n_geo) {
 }
 
 __global__ void radii_scatter_kernel(const PairRec* __restrict__ pairs, const int* __restrict__ n_pair,
-                                     int* __restrict__ hist, int n_geo, int* __restrict__ order) {
+                                     const int* __restrict__ rank, int* __restrict__ hist, int n_geo, int* __restrict__ order) {
     const int np = *n_pair;
     for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < np; p += gridDim.x * blockDim.x)
-        order[atomicAdd(hist + n_geo + pairs[p].geo, 1)] = p;
+        order[atomicAdd(hist + n_geo + (rank ? rank[pairs[p].geo] : pairs[p].geo), 1)] = p;
 }
 
 // The radius classes of the sorted order: after the scatter, hist[n_geo + g]
@@ -229,8 +230,8 @@ __global__ void radii_classes_kernel(const int* __restrict__ hist, int n_geo, in
     }
 }
 
-// The same for ranges of geometries (class k takes range[k].x .. range[k].y):
-// the runs are adjacent in the order, the largest geometry first.
+// The same for ranges of ranks (class k takes range[k].x .. range[k].y):
+// the runs are adjacent in the order, the highest rank first.
 __global__ void class_runs_kernel(const int* __restrict__ hist, int n_geo, const int2* __restrict__ range, int n_class,
                                   int* __restrict__ cls) {
     const int k = threadIdx.x;
@@ -370,12 +371,12 @@ cudaError_t launch_pair_list_packed(int n, const double* centers, const double L
 }
 
 cudaError_t launch_radii_sort(const PairRec* pairs, const int* n_pair, int* hist, int n_geo, int* order, int num_sms,
-                              cudaStream_t st, int* classes) {
+                              cudaStream_t st, int* classes, const int* rank) {
     cudaError_t e = cudaMemsetAsync(hist, 0, sizeof(int) * 2 * n_geo, st);
     if (e != cudaSuccess) return e;
-    radii_count_kernel<<<num_sms * 2, 256, 0, st>>>(pairs, n_pair, hist, n_geo);
+    radii_count_kernel<<<num_sms * 2, 256, 0, st>>>(pairs, n_pair, rank, hist, n_geo);
     radii_scan_kernel<<<1, 32, 0, st>>>(hist, n_geo);
-    radii_scatter_kernel<<<num_sms * 2, 256, 0, st>>>(pairs, n_pair, hist, n_geo, order);
+    radii_scatter_kernel<<<num_sms * 2, 256, 0, st>>>(pairs, n_pair, rank, hist, n_geo, order);
     if (classes) radii_classes_kernel<<<1, 64, 0, st>>>(hist, n_geo, classes);
     return cudaGetLastError();
 }

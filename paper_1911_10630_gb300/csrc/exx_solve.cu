@@ -76,6 +76,18 @@ __device__ int cg_ball(T* __restrict__ pc, T* __restrict__ r, T* __restrict__ d,
     return it;
 }
 
+// This thread's share of a.b over k < n as one of 256 threads (0 for the others);
+// b is indexed through cube when that is given.
+template <typename T>
+__device__ __forceinline__ T sum256(const T* a, const T* b, const int* cube, int n) {
+    T acc = T(0);
+    if (threadIdx.x < 256) {
+#pragma unroll 8
+        for (int k = threadIdx.x; k < n; k += 256) acc = fma(a[k], b[cube ? __ldg(cube + k) : k], acc);
+    }
+    return acc;
+}
+
 // PCG on the PE ball with the V-cycle as the preconditioner. On entry: r = rhs,
 // d = 0, rr = ||rhs||^2; p goes to the cube pc (zero off the ball). Returns
 // the iteration count; rr_out receives the final recursive ||r||^2.
@@ -84,8 +96,10 @@ __device__ int cg_ball(T* __restrict__ pc, T* __restrict__ r, T* __restrict__ d,
 //   recurrence and the V-cycle in FP32 on the normalised residual, the stop
 //   test of the refinement loop on the FP64 residual.
 // Inlined into the kernel with P its own parameter block, so that the sweeps
-// read the level operators as parameter constants; U unrolls the sweeps.
-template <int NT, typename T, int U>
+// read the level operators as parameter constants; U unrolls the sweeps. SPLIT:
+// the sums are taken apart from the sweeps by 256 of the threads (sum256), so that
+// they are those of 256 threads bit for bit.
+template <int NT, typename T, int U, bool SPLIT>
 __device__ __forceinline__ int mg_pcg(const SolveParams& P, const BallGeo& G, const MGGeo& M, char* slot,
                                       T* __restrict__ pc, T* __restrict__ r, T* __restrict__ d, T* __restrict__ ap, T rr,
                                       T target2, int max_iter, T (*red)[33], int& flip, T& rr_out) {
@@ -96,7 +110,9 @@ __device__ __forceinline__ int mg_pcg(const SolveParams& P, const BallGeo& G, co
     const T* __restrict__ Z = reinterpret_cast<const T*>(slot + P.off_tc);  // z = M r (level-0 cube)
     T* __restrict__ Zj = reinterpret_cast<T*>(slot + P.off_zc);             // the V-cycle's first Jacobi sweep
     const T wd = mg_wd<T>(P, 0);
-    T rz = block_sum<NT, T>(mg_vcycle<NT, T, U>(P, G, M, slot, r), red, flip);
+    T rz = mg_vcycle<NT, T, U>(P, G, M, slot, r);
+    if (SPLIT) rz = sum256(r, Z, cube, n_pe);
+    rz = block_sum<NT, T>(rz, red, flip);
     for (int k = threadIdx.x; k < n_pe; k += NT) {
         const int c = cube[k];
         pc[c] = Z[c];
@@ -110,7 +126,11 @@ __device__ __forceinline__ int mg_pcg(const SolveParams& P, const BallGeo& G, co
             const int c = cube[k];
             const T a = lap19<T>(pc, c, S, S2, A);
             ap[k] = a;
-            pap = fma(pc[c], a, pap);
+            if (!SPLIT) pap = fma(pc[c], a, pap);
+        }
+        if (SPLIT) {
+            __syncthreads();
+            pap = sum256(ap, pc, cube, n_pe);
         }
         pap = block_sum<NT, T>(pap, red, flip);
         const T al = rz / pap;
@@ -123,13 +143,19 @@ __device__ __forceinline__ int mg_pcg(const SolveParams& P, const BallGeo& G, co
             const T rk = fma(-al, ap[k], r[k]);
             r[k] = rk;
             Zj[c] = wd * rk;
-            rrn = fma(rk, rk, rrn);
+            if (!SPLIT) rrn = fma(rk, rk, rrn);
+        }
+        if (SPLIT) {
+            __syncthreads();
+            rrn = sum256(r, r, nullptr, n_pe);
         }
         rrn = block_sum<NT, T>(rrn, red, flip);
         ++it;
         rr = rrn;
         if (rrn <= target2 || !(rrn == rrn)) break;
-        const T rzn = block_sum<NT, T>(mg_vcycle<NT, T, U>(P, G, M, slot, r, 0, true), red, flip);
+        T rzn = mg_vcycle<NT, T, U>(P, G, M, slot, r, 0, true);
+        if (SPLIT) rzn = sum256(r, Z, cube, n_pe);
+        rzn = block_sum<NT, T>(rzn, red, flip);
         const T be = rzn / rz;
         rz = rzn;
 #pragma unroll (U)
@@ -155,11 +181,16 @@ __device__ __forceinline__ int mg_pcg(const SolveParams& P, const BallGeo& G, co
 // Measured on one box, water-64 workload: five 0.512 s (unrolled) / 0.507
 // (not), six 0.488 (unrolled); batched-uneven workload: five 0.331 / 0.328,
 // six 0.467 (unrolled).
-template <int NT, bool ONE_BALL>
-constexpr int mg_min_blocks() { return NT == 256 ? (ONE_BALL ? 6 : 5) : 1024 / NT; }
+// FEW: no more pairs than two CTAs per SM hold. 512 threads to a pair, the sums in
+// the order of 256 (see march_steady in exx_api.cu for what another order does to
+// the balls that come here): the same results bit for bit, 269 pairs at R_PE 19 and 25 in 27 ms (42 with 256
+// threads). For many pairs 256 threads and five CTAs per SM stay the better form
+// (512 orbitals with radii of 12 to 29: 292 ms, 326 with 512).
+template <int NT, bool ONE_BALL, bool FEW>
+constexpr int mg_min_blocks() { return FEW ? 2 : NT == 256 ? (ONE_BALL ? 6 : 5) : 1024 / NT; }
 
-template <int NT, bool MIXED, bool MG = false, bool ONE_BALL = false>
-__global__ void __launch_bounds__(NT, MG ? mg_min_blocks<NT, ONE_BALL>() : (MIXED ? 1 : 2)) pair_kernel(const __grid_constant__ SolveParams P) {
+template <int NT, bool MIXED, bool MG = false, bool ONE_BALL = false, bool FEW = false>
+__global__ void __launch_bounds__(NT, MG ? mg_min_blocks<NT, ONE_BALL, FEW>() : (MIXED ? 1 : 2)) pair_kernel(const __grid_constant__ SolveParams P) {
     extern __shared__ double smem[];
     __shared__ double red[2][33];
     __shared__ float red32[2][33];
@@ -167,6 +198,8 @@ __global__ void __launch_bounds__(NT, MG ? mg_min_blocks<NT, ONE_BALL>() : (MIXE
     __shared__ int s_item;
     __shared__ double s_ub[NT / 32][kNU + kNU / 2];
     int flip = 0, flip32 = 0;
+
+    if (MG && MIXED && (FEW || NT == 256) && (*P.n_pair <= P.few) != FEW) return;  // the other form's
 
     const int Rc = P.Rc;
     const int S = P.S;
@@ -212,7 +245,12 @@ __global__ void __launch_bounds__(NT, MG ? mg_min_blocks<NT, ONE_BALL>() : (MIXE
         long long tr = 0;
 
         // 1. gather rho on the PE ball; v = 0 there
-        gather_rho(P, G, pr, rho, vc, threadIdx.x, NT);
+        if constexpr (FEW) {
+            if (P.box_org) (void)gather_wide<true>(P, G, pr, rho, vc, threadIdx.x, NT);
+            else (void)gather_wide<false>(P, G, pr, rho, vc, threadIdx.x, NT);
+        } else {
+            gather_rho(P, G, pr, rho, vc, threadIdx.x, NT);
+        }
         __syncthreads();
 
         // 2. multipole moments and polynomial coefficients
@@ -243,7 +281,7 @@ __global__ void __launch_bounds__(NT, MG ? mg_min_blocks<NT, ONE_BALL>() : (MIXE
             double rr_fin;
             const double target2 = P.tol * P.tol * bb;
             if (MG && P.mg[pr.geo].L > 0)
-                iters = mg_pcg<NT, double, 2>(P, G, P.mg[pr.geo], slot, pc, r, d, ap, bb, target2, P.max_iter, red,
+                iters = mg_pcg<NT, double, 2, false>(P, G, P.mg[pr.geo], slot, pc, r, d, ap, bb, target2, P.max_iter, red,
                                            flip, rr_fin);
             else
                 iters = cg_ball<double, NT>(pc, r, d, ap, cube, n_pe, S, S2, neg64, bb, target2, P.max_iter, red,
@@ -257,12 +295,17 @@ __global__ void __launch_bounds__(NT, MG ? mg_min_blocks<NT, ONE_BALL>() : (MIXE
                 // FP64 residual r = 4 pi rho + lap v (v: current iterate on PE, shell values outside)
                 const long long tu = clk ? clock64() : 0;
                 double acc = 0.0;
+#pragma unroll (FEW ? 2 : 1)
                 for (int k = threadIdx.x; k < n_pe; k += NT) {
                     const int c = cube[k];
                     const double rk = fma(four_pi, rho[k], lap19<double>(vc, c, S, S2, P.st64));
                     r[k] = rk;
-                    acc = fma(rk, rk, acc);
+                    if (!FEW) acc = fma(rk, rk, acc);
                     if (bb < 0.0 && P.dbg_b) P.dbg_b[k] = rk;
+                }
+                if (FEW) {
+                    __syncthreads();
+                    acc = sum256(r, r, nullptr, n_pe);
                 }
                 const double rn2 = block_sum<NT, double>(acc, red, flip);
                 if (clk) tr += clock64() - tu;
@@ -282,7 +325,11 @@ __global__ void __launch_bounds__(NT, MG ? mg_min_blocks<NT, ONE_BALL>() : (MIXE
                     r32[k] = rk;
                     p32[c] = rk;
                     d32[k] = 0.0f;
-                    acc32 = fmaf(rk, rk, acc32);
+                    if (!FEW) acc32 = fmaf(rk, rk, acc32);
+                }
+                if (FEW) {
+                    __syncthreads();
+                    acc32 = sum256(r32, r32, nullptr, n_pe);
                 }
                 const float rr32 = block_sum<NT, float>(acc32, red32, flip32);
                 double eta = 0.3 * P.tol * sqrt(bb) / rn;
@@ -290,7 +337,7 @@ __global__ void __launch_bounds__(NT, MG ? mg_min_blocks<NT, ONE_BALL>() : (MIXE
                 float rr_fin;
                 const int budget = min(P.inner_max_iter, P.max_iter - iters);
                 if (MG && P.mg[pr.geo].L > 0)
-                    iters += mg_pcg<NT, float, ONE_BALL ? 2 : 1>(P, G, P.mg[pr.geo], slot, p32, r32, d32, ap32, rr32,
+                    iters += mg_pcg<NT, float, FEW || ONE_BALL ? 2 : 1, FEW>(P, G, P.mg[pr.geo], slot, p32, r32, d32, ap32, rr32,
                                                (float)(eta * eta) * rr32, budget, red32, flip32, rr_fin);
                 else
                     iters += cg_ball<float, NT>(p32, r32, d32, ap32, cube, n_pe, S, S2, neg32, rr32,
@@ -313,7 +360,8 @@ __global__ void __launch_bounds__(NT, MG ? mg_min_blocks<NT, ONE_BALL>() : (MIXE
             if (P.refines) P.refines[pidx] = refines;
             if (!conv) atomicAdd(P.nonconv, 1);
         }
-        scatter_dxx(P, G, pr, vc, threadIdx.x, NT);
+        if constexpr (FEW) scatter_wide(P, G, pr, vc, threadIdx.x, NT);
+        else scatter_dxx(P, G, pr, vc, threadIdx.x, NT);
         if (P.n_geo > 1) {
             // the next pair may have another ball: the direction cube must be
             // zero outside it, so clear the points this pair wrote
@@ -386,9 +434,11 @@ size_t pair_kernel_smem(int Rc, int r_pe_max) {
 
 cudaError_t launch_pair_kernel(const SolveParams& P, int threads, bool mixed, int grid, size_t smem, cudaStream_t st) {
     if (P.mg) {  // the multigrid-preconditioned CG: FP64, or FP32 inside FP64 refinement
-        if (!mixed) pair_kernel<512, false, true><<<grid, 512, smem, st>>>(P);
-        else if (threads == 256 && P.n_geo == 1) pair_kernel<256, true, true, true><<<grid, 256, smem, st>>>(P);
-        else if (threads == 256) pair_kernel<256, true, true><<<grid, 256, smem, st>>>(P);
+        if (mixed && threads == 256) {  // both forms: the device knows how many pairs there are
+            if (P.n_geo == 1) pair_kernel<256, true, true, true><<<grid, 256, smem, st>>>(P);
+            else pair_kernel<256, true, true><<<grid, 256, smem, st>>>(P);
+            if (P.few > 0) pair_kernel<512, true, true, false, true><<<grid < P.few ? grid : P.few, 512, smem, st>>>(P);
+        } else if (!mixed) pair_kernel<512, false, true><<<grid, 512, smem, st>>>(P);
         else if (threads == 1024) pair_kernel<1024, true, true><<<grid, 1024, smem, st>>>(P);
         else pair_kernel<512, true, true><<<grid, 512, smem, st>>>(P);
         return cudaGetLastError();
@@ -411,6 +461,9 @@ cudaError_t pair_kernel_occupancy(int threads, bool mixed, bool mg, bool one_bal
     else if (threads == 1024) f = (const void*)pair_kernel<1024, true>;
     else f = (const void*)pair_kernel<512, true>;
     cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e == cudaSuccess && mg && mixed && threads == 256)
+        e = cudaFuncSetAttribute((const void*)pair_kernel<512, true, true, false, true>,
+                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, f, threads, smem);
 }

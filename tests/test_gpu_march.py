@@ -1,8 +1,9 @@
 """The FP32 multigrid CG's marching kernel against the general FP64 kernel (same
 hierarchy, FP64 throughout) at the sizes where its layout changes: the smallest
 balls with a coarse level; odd and even radii; the last ball of 128, 256 and 512
-columns and the first beyond (16/17, 24/25, 34/35: the last runs on the general
-kernel); CTA sizes chosen by the caller; two classes of CTA size in one call;
+columns and the first beyond (16/20, 24/28, 34/35); balls that
+stay on the general kernel in FP32 (9, 13, 17, 21, 25, 33 to 35), alone, few and
+many, and beside others; CTA sizes chosen by the caller; two classes of CTA size in one call;
 anisotropic ragged grids (FP64 stencil residuals); the integer residual and its
 overflow fallback.
 
@@ -25,7 +26,8 @@ def torch():
 
 # R_PE, R_PE of the non-self pairs (0: the same), anisotropic, options
 CASES = [(4, 0, 0, {}), (5, 0, 1, {}), (8, 0, 0, {}), (9, 0, 0, {}), (13, 0, 0, {}), (16, 0, 0, {}), (17, 0, 1, {}),
-         (24, 0, 0, {}), (25, 0, 0, {}), (33, 0, 0, {}), (34, 0, 0, {}), (35, 0, 0, {}),
+         (24, 0, 0, {}), (10, 0, 0, {}), (11, 0, 1, {}), (12, 0, 0, {}), (15, 0, 0, {}), (20, 0, 0, {}), (28, 0, 1, {}),
+         (31, 0, 0, {}), (32, 0, 0, {}), (30, 21, 0, {}), (21, 12, 0, {}), (25, 0, 0, {}), (33, 0, 0, {}), (34, 0, 0, {}), (35, 0, 0, {}),
          (16, 0, 0, dict(threads=256)), (17, 0, 0, dict(threads=512)), (9, 0, 1, dict(threads=1024)),
          (24, 0, 0, dict(threads=1024)), (25, 12, 0, {}), (18, 13, 1, {}), (16, 5, 0, dict(ctas_per_sm=1)),
          (20, 0, 0, dict(fixed_residual=1)), (20, 12, 0, dict(fixed_residual=2))]
