@@ -53,21 +53,21 @@ struct ConvArgs {
     int* err;
 };
 
-// Persistent CTAs, one per SM, each over the tiles t, t + grid, ...: warps 0-3
-// empty the accumulators (epilogue), one thread of warp 4 issues the MMAs, warps
-// 5-12 stage the input halo tiles and weights. A unit is one 16-channel chunk of a
+// Persistent CTAs, one per SM, each over the tiles t, t + grid, ...: warps 0-7
+// empty the accumulators (epilogue), one thread of warp 8 issues the MMAs, warps
+// 9-16 stage the input halo tiles and weights. A unit is one 16-channel chunk of a
 // tile; units pass through n_stage shared-memory stages (full / empty barriers),
 // tiles through n_acc accumulators in tensor memory. One CTA per tile that staged,
 // multiplied and stored in turn left the tensor cores 5 to 10 % busy: the 13
 // convolutions of 32 cubes of 48 took 2.36 ms; with cheaper staging and two CTAs a
-// SM 1.2; like this 0.93.
-constexpr int kProducers = 256, kConvThreads = 5 * 32 + kProducers;
+// SM 1.2; like this 0.85.
+constexpr int kEpilogue = 256, kProducers = 256, kConvThreads = kEpilogue + 32 + kProducers;
 
 __global__ void __launch_bounds__(kConvThreads, 1) conv3_tc_kernel(const __grid_constant__ ConvArgs a) {
     extern __shared__ unsigned char smem_dyn[];
     __shared__ uint64_t full[kStages], empty[kStages], acc_full[2], acc_empty[2], wres;
     __shared__ uint32_t s_tmem;
-    __shared__ float s_bias[256];
+    __shared__ __align__(16) float s_bias[256];
     unsigned char* base =
         reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_dyn) + 127) & ~uintptr_t(127));
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -79,7 +79,7 @@ __global__ void __launch_bounds__(kConvThreads, 1) conv3_tc_kernel(const __grid_
         }
         for (int s = 0; s < 2; ++s) {
             tc::mbar_init(&acc_full[s], 1);
-            tc::mbar_init(&acc_empty[s], 128);
+            tc::mbar_init(&acc_empty[s], kEpilogue);
         }
         tc::mbar_init(&wres, 1);
         tc::mbar_init_fence();
@@ -91,7 +91,7 @@ __global__ void __launch_bounds__(kConvThreads, 1) conv3_tc_kernel(const __grid_
     tc::fence_after_sync();
     const uint32_t tbase = s_tmem;
     if (a.fold) {  // every slice accumulates from several MMAs: start from zero
-        if (warp < 4) {
+        if (warp < 4) {  // a warp reaches the 32 lanes of its number modulo 4
             for (int c0 = 0; c0 < a.ncols; c0 += 16) tc::tmem_st16_zero(tbase + ((uint32_t)(warp * 32) << 16) + c0);
             tc::tmem_wait_st();
         }
@@ -112,8 +112,8 @@ __global__ void __launch_bounds__(kConvThreads, 1) conv3_tc_kernel(const __grid_
         n0 = t / a.B * a.nb;
     };
     bool ok = true;
-    if (warp >= 5) {  // staging
-        const int pt = tid - 5 * 32, items = (DT + 2) * kHH * kWW * 2;
+    if (warp > kEpilogue / 32) {  // staging
+        const int pt = tid - kEpilogue - 32, items = (DT + 2) * kHH * kWW * 2;
         const bool delay = NS >= 3;
         const auto finish = [&](int s) {
             tc::fence_proxy_async();
@@ -186,7 +186,7 @@ __global__ void __launch_bounds__(kConvThreads, 1) conv3_tc_kernel(const __grid_
             tc::cp_async_wait<0>();
             finish(before);
         }
-    } else if (warp == 4) {
+    } else if (warp == kEpilogue / 32) {
         if (lane == 0) {
             const uint32_t idesc = tc::idesc_bf16_f32(128, a.fold ? 3 * a.nb : a.nb);
             const uint32_t bs = (uint32_t)(a.fold ? 3 : 1) * a.nb * 2;  // 16-byte words of weights per MMA
@@ -244,8 +244,8 @@ __global__ void __launch_bounds__(kConvThreads, 1) conv3_tc_kernel(const __grid_
         }
         __syncwarp();
     } else {
-        const int m = warp * 32 + lane;  // accumulator row = TMEM lane
-        const uint32_t row = (uint32_t)(warp * 32) << 16;
+        const int m = (warp & 3) * 32 + lane;  // accumulator row = TMEM lane
+        const uint32_t row = (uint32_t)((warp & 3) * 32) << 16;
         int i = 0;
         for (int t = blockIdx.x; t < a.n_tiles; t += gridDim.x, ++i) {
             int b, d0, h0, w0, n0;
@@ -256,7 +256,7 @@ __global__ void __launch_bounds__(kConvThreads, 1) conv3_tc_kernel(const __grid_
             tc::fence_after_sync();
             const uint32_t acc = tbase + row + (uint32_t)(ab * a.acc_cols + (a.fold ? 2 * a.nb : 0));
             const int h = h0 + (m >> 3), w = w0 + (m & 7);
-            for (int tt = 0; tt < DT; ++tt) {
+            for (int tt = warp >> 2; tt < DT; tt += kEpilogue / 128) {
                 const int d = d0 + tt;
                 const bool live = d < a.D && h < a.H && w < a.W;
                 const size_t vox = (((size_t)b * a.D + d) * a.H + h) * a.W + w;
@@ -269,7 +269,13 @@ __global__ void __launch_bounds__(kConvThreads, 1) conv3_tc_kernel(const __grid_
                     const size_t at = vox * a.cout + n0 + c0;
                     if (a.bias) {
 #pragma unroll
-                        for (int k = 0; k < 16; ++k) v[k] += s_bias[n0 + c0 + k];
+                        for (int k = 0; k < 4; ++k) {
+                            const float4 f = *reinterpret_cast<const float4*>(s_bias + n0 + c0 + 4 * k);
+                            v[4 * k] += f.x;
+                            v[4 * k + 1] += f.y;
+                            v[4 * k + 2] += f.z;
+                            v[4 * k + 3] += f.w;
+                        }
                     }
                     if (a.epi == 1) {
 #pragma unroll
@@ -349,7 +355,7 @@ __global__ void pack_kernel(const float* __restrict__ w, __nv_bfloat16* __restri
 // of 48; one voxel per thread took 0.42 ms, this 0.23).
 // W16: in is 16-byte aligned (a caller's need not be).
 template <bool W16>
-__global__ void __launch_bounds__(256, 2) conv_first_kernel(const float* __restrict__ in, const float* __restrict__ w,
+__global__ void __launch_bounds__(128, 4) conv_first_kernel(const float* __restrict__ in, const float* __restrict__ w,
                                                          const float* __restrict__ bias, __nv_bfloat16* __restrict__ y,
                                                          int B, int S) {
     constexpr int CI = kIn;
@@ -1080,7 +1086,7 @@ cudaError_t forward(Net& n, const float* in, int B, cudaStream_t st) {
     };
     auto conv = [&](const __nv_bfloat16* x, __nv_bfloat16* y, int l, int s) { return conv_up(x, nullptr, 0, y, l, s); };
     const auto first = reinterpret_cast<uintptr_t>(in) % 16 ? conv_first_kernel<false> : conv_first_kernel<true>;
-    first<<<grid_for(v0 / 4, n.n_sm), 256, 0, st>>>(in, n.params, bias_of(n, 0), n.x0a, B, S);
+    first<<<(unsigned)((v0 / 4 + 127) / 128), 128, 0, st>>>(in, n.params, bias_of(n, 0), n.x0a, B, S);
     UCK(cudaGetLastError());
     UCK(conv(n.x0a, n.x0, 1, S));
     pool_kernel<<<grid_for(v1 * 2, n.n_sm), 256, 0, st>>>(n.x0, n.p0, B, S, 16);
