@@ -37,12 +37,15 @@ SMEM_BYTES_PER_CLK_SM = 128  # shared-memory bandwidth of one SM (32 banks x 4 B
 # loads of 16 bytes per quad of 4 points plus the store of p (context only;
 # the roofline's algorithmic bytes are the CG state's)
 SMEM_MODEL_BYTES_PER_POINT_ITER = 15 * 16 / 4 + 4
-# The multigrid PCG's algorithmic bytes per fine-level point and iteration
-# (FP32, every vector read or written once per sweep): A p (8), the d and r
-# updates (24), the V-cycle's level-0 sweeps: Jacobi (8), residual (12),
-# restriction (4), prolongation (8), smoothing (12); r.z (8) and the p update
-# (12): 96 B; the coarse levels add their share of the V-cycle (44 B x 1/7)
-MG_BYTES_PER_POINT_ITER = 96 + 44 / 7
+# The multigrid PCG's algorithmic bytes per fine-level point and iteration (FP32,
+# every vector once per pass): z, p and d read and p, d and A p written (24), r and
+# A p read and r written (12), r read and z written (8): 44 B; the coarse levels add
+# their share of the V-cycle (44 B x 1/7)
+MG_BYTES_PER_POINT_ITER = 44 + 44 / 7
+# The plain FP64 CG's: A p reads p and its fixed-point copy and writes q (24), the
+# residual reads q and r and writes r (24), the direction reads r, x and p and writes
+# x, p and the copy (48); four bytes of index per pair of points in two of them (4)
+FP64_BYTES_PER_POINT_ITER = 24 + 24 + 48 + 4
 
 
 def _peaks():
@@ -58,7 +61,7 @@ def _peaks():
 # the sources that decide the pair kernels' code and launch layout (DRAM
 # traffic): a change to any of them invalidates the committed ncu figures
 KERNEL_SOURCES = ("exx_cluster.cu", "exx_phases.cuh", "exx_kernels.cuh", "exx_internal.h", "exx_geometry.cpp",
-                  "exx_geometry.h", "exx_solve.cu", "exx_mg.cuh")
+                  "exx_geometry.h", "exx_solve.cu", "exx_mg.cuh", "exx_march.cu", "exx_march.cuh", "exx_cg64.cu")
 
 
 def _kernel_hash():
@@ -443,24 +446,32 @@ def main():
                         "achieved": alg_["hbm"] / (kms / 1e3) / 1e9, "peak": hbm_peak, "peak_source": peak_src},
                 "kernel_ms": kms}
 
+    def fp64_roofline(alg_, kms):
+        """The plain FP64 CG's: A p in integers leaves its vectors' bytes as the bound."""
+        nbytes = FP64_BYTES_PER_POINT_ITER * alg_["point_iters"]
+        achieved = nbytes / (kms / 1e3) / 1e9
+        return {"kernel": "cg64_kernel", "bound": "hbm", "achieved": achieved, "peak": hbm_peak, "unit": "GB/s",
+                "frac": achieved / hbm_peak, "peak_source": peak_src, "algorithmic_bytes_per_launch": nbytes,
+                "bytes_per_point_iteration": FP64_BYTES_PER_POINT_ITER,
+                "traffic": _traffic("cg64_kernel", f"{w.name}|p0"),
+                "equivalent_fp64": {"flops_per_point_iteration": 38, "achieved": alg_["flops"] / (kms / 1e3) / 1e12,
+                                    "peak": fp64_peak, "unit": "TFLOP/s",
+                                    "peak_source": "FP64 FMA rate measured on this GPU (exx_probe_fp64_rate)"},
+                "kernel_ms": kms}
+
     if args.precision == 1 and args.preconditioner == 1:
-        # one CTA per pair, every vector in the pair's workspace: the sweeps
+        # one CTA per pair, every vector in the pair's workspace: the passes
         # stream from HBM (the pairs in flight hold far more than L2)
         mg_bytes = MG_BYTES_PER_POINT_ITER * alg["point_iters"]
         achieved = mg_bytes / (kern_ms / 1e3) / 1e9
-        roofline = {"kernel": "pair_kernel", "bound": "hbm", "achieved": achieved, "peak": hbm_peak, "unit": "GB/s",
+        roofline = {"kernel": "march_kernel", "bound": "hbm", "achieved": achieved, "peak": hbm_peak, "unit": "GB/s",
                     "frac": achieved / hbm_peak, "peak_source": peak_src,
                     "algorithmic_bytes_per_launch": mg_bytes, "bytes_per_point_iteration": MG_BYTES_PER_POINT_ITER,
-                    "traffic": _traffic("pair_kernel", workload_key), "kernel_ms": kern_ms}
+                    "traffic": _traffic("march_kernel", workload_key), "kernel_ms": kern_ms}
     elif args.precision == 1:
         roofline = cg_roofline(st, alg, kern_ms)
     else:
-        fl = alg["flops"] / (kern_ms / 1e3) / 1e12
-        roofline = {"kernel": "pair_kernel", "bound": "alu", "achieved": fl, "peak": fp64_peak,
-                    "unit": "TFLOP/s", "frac": fl / fp64_peak,
-                    "peak_source": "FP64 FMA rate measured on this GPU (exx_probe_fp64_rate)",
-                    "flops_per_point_iteration": 38, "traffic": _traffic("pair_kernel", workload_key),
-                    "kernel_ms": kern_ms}
+        roofline = fp64_roofline(alg, kern_ms)
 
     # the host-buffer leg runs first, before the comparison contexts below
     # allocate and free their workspaces (measured: copies into freshly
@@ -500,17 +511,11 @@ def main():
             t.append(ev0.elapsed_time(ev1))
         st0 = ex0.stats()
         alg0 = _algorithmic(ex0.pairs(), st0, n_pe, n_me, 0)
-        fl0 = alg0["flops"] / (st0["solve_ms"] / 1e3) / 1e12
         extra["plain_fp64_cg"] = {"value": n_pair / (statistics.mean(t) / 1e3), "unit": UNIT,
                                   "ms_per_step": statistics.mean(t), "E_xx": e0,
                                   "dE_vs_fast_per_orbital": abs(e0 - exx_vals[-1]) / w.n,
                                   "iters_p50": st0["iters_p50"], "iters_max": st0["iters_max"],
-                                  "roofline": {"kernel": "pair_kernel", "bound": "alu", "achieved": fl0,
-                                               "peak": fp64_peak, "unit": "TFLOP/s", "frac": fl0 / fp64_peak,
-                                               "peak_source": "FP64 FMA rate measured on this GPU "
-                                                              "(exx_probe_fp64_rate)",
-                                               "flops_per_point_iteration": 38,
-                                               "kernel_ms": st0["solve_ms"]}}
+                                  "roofline": fp64_roofline(alg0, st0["solve_ms"])}
         extra["speedup_vs_plain_fp64_cg"] = value / ws / extra["plain_fp64_cg"]["value"]
         ex0.close()
         if args.preconditioner == 1:

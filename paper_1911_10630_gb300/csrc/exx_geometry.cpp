@@ -178,8 +178,9 @@ void build_ball(HostBall& B, int r_pe, int r_me, int Rc) {
     B.n_me = (int)B.cube.size();
 }
 
-// The PE ball's rim first, and the shell layer that its stencils read with 1 / r.
-void build_ball_layers(HostBall& B, int Rc, const double delta[3]) {
+// The PE ball's rim first, the shell layer that its stencils read with 1 / r, and
+// (duos) the ball's points in pairs.
+void build_ball_layers(HostBall& B, int Rc, const double delta[3], bool duos) {
     B.rim.clear();
     const int in2 = B.r_pe > 3 ? (B.r_pe - 3) * (B.r_pe - 3) : -1;
     for (int pass = 0; pass < 2; ++pass) {
@@ -192,7 +193,7 @@ void build_ball_layers(HostBall& B, int Rc, const double delta[3]) {
     B.duo.clear();
     B.duo_k.clear();
     const int S = 2 * Rc + 1;
-    for (int lo = -B.r_pe; lo <= B.r_pe; lo += kBand)
+    for (int lo = -B.r_pe; duos && lo <= B.r_pe; lo += kBand)
         for (const RowRec& R : B.rows_pe) {
             if (R.oy < lo || R.oy >= lo + kBand) continue;
             const int c0 = ((R.ox + Rc) * S + (R.oy + Rc)) * (S + 1), z0 = Rc - R.zpe, z1 = Rc + R.zpe;

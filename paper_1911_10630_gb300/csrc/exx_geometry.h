@@ -18,7 +18,7 @@ struct HostBall {
     std::vector<int> sh_near;       // shell points with |z| <= zn of their ME row: row << 8 | (z + 128)
     std::vector<int> sh_far;        // the other shell points, same packing
     std::vector<int> rim;           // PE points whose stencils reach the shell (n_rim), then the others
-    int n_rim;
+    int n_rim = 0;
     std::vector<int> layer;         // shell points that the stencil reads: ME row << 8 | |z|
     std::vector<double> layer_ir;   // and their 1 / r
     std::vector<int> duo, duo_k;    // PE points in pairs along z, by bands of kBand rows in y
@@ -35,7 +35,7 @@ void build_multipole_const(MultipoleConst& mc);
 bool build_cluster_layout(const HostBall& B, int C, ClusterLayout& L, std::vector<int>& pt_slab, bool pitch4 = false,
                           int max_planes = 0);
 void build_ball(HostBall& B, int r_pe, int r_me, int Rc);
-void build_ball_layers(HostBall& B, int Rc, const double delta[3]);
+void build_ball_layers(HostBall& B, int Rc, const double delta[3], bool duos);
 
 // Thread-slot maps of the cluster solver for NT threads x PTS points per CTA:
 // slot (j, t) of CTA r holds one point of the CTA's slab. Points are dealt so
