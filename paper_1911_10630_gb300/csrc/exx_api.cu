@@ -1297,11 +1297,14 @@ extern "C" exx_status exx_init(exx_ctx** out, const double cell[3], const int gr
     const double W[4] = {-49.0 / 18.0, 3.0 / 2.0, -3.0 / 20.0, 1.0 / 90.0};  // Eq. d2_1
     double inv2[3];
     for (int a = 0; a < 3; ++a) inv2[a] = 1.0 / (c->delta[a] * c->delta[a]);
-    // isotropic grids: 180 delta^2 x the weights are the integers -490, 270, -27, 2
-    P.fixres = (isotropic(c) && c->opt.fixed_residual != 1)
+    // isotropic grids: 180 delta^2 x the weights are the integers -490, 270, -27, 2.
+    // The cluster solver takes equal spacings only: its CG carries a last-bit
+    // difference of the operator up to 1e-9 of D_xx.
+    const bool equal = c->delta[0] == c->delta[1] && c->delta[1] == c->delta[2];
+    P.fixres = ((c->march.empty() ? equal : isotropic(c)) && c->opt.fixed_residual != 1)
                    ? (c->opt.fixed_residual == 2 ? 2 : 1)
                    : 0;
-    P.fix_inv = (inv2[0] + inv2[1] + inv2[2]) / 540.0;
+    P.fix_inv = equal ? inv2[0] / 180.0 : (inv2[0] + inv2[1] + inv2[2]) / 540.0;
     P.dfix = c->opt.deterministic ? 1099511627776.0 : 0.0;  // 2^40
     P.st64.c0 = W[0] * (inv2[0] + inv2[1] + inv2[2]);
     for (int q = 1; q <= 3; ++q) {
