@@ -274,6 +274,7 @@ __global__ void __launch_bounds__(NT, 1024 / NT) cg64_kernel(const __grid_consta
     const int np = *P.n_pair;
     const bool lead = rank == 0 && tid == 0;
 
+    team_sync(C);  // every CTA of the team has started: its shared memory may be written
     for (;;) {
         if (lead) {
             const int i = atomicAdd(P.queue, 1);

@@ -1660,6 +1660,7 @@ __global__ void __launch_bounds__(NT, MINB) cluster_mg_kernel(const __grid_const
     const int gt = rank * NT + t, gn = C * NT;
     const int np = *P.n_pair;
 
+    cl.sync();  // every CTA of the cluster has started: its shared memory may be written
     for (;;) {
         if (rank == 0 && t == 0) {
             const int it = atomicAdd(P.queue, 1);
