@@ -62,7 +62,7 @@ struct PairState {
     int fix;               // the FP64 residuals come from the fixed-point copy of v
     int ovf;               // a value of v did not fit it
     double bb, rn_prev;
-    double scale;          // the PCG's right-hand side over the residual: a power of 2
+    double scale;          // the PCG's right-hand side over the residual: a power of 2 (exact)
     double s2E, finvE;     // fixed-point scale of v, and of its integer stencil's sums
     double vnear;          // largest |v| on the shell layer that the stencil reads
     long long clk[3], tr;
@@ -366,9 +366,13 @@ __global__ void __launch_bounds__(NT, MINB) march_kernel(const __grid_constant__
             __syncthreads();
             if (threadIdx.x == 0) {
                 if (S.ovf) S.fix = S.ovf = 0;  // beyond the copy's range: the FP64 stencil from here on
-                int e = 0;  // the next residual is smaller by about eta
-                (void)frexp(eta, &e);
-                if (S.scale < 1e280) S.scale = ldexp(S.scale, -e);
+                // The next residual's norm lies between eta times this one's and, where the
+                // inner solve stopped short, this one's: with eta at 2^-24 or more (what FP32
+                // can gain) its squares stay within FP32's range. From the residual itself,
+                // not from the last scale: solves that keep stopping short do not add up.
+                int e = 0;
+                (void)frexp(rn * fmax(eta, 5.9604644775390625e-8), &e);
+                S.scale = ldexp(1.0, -min(max(e, -900), 900));
             }
             __syncthreads();
         }
