@@ -385,6 +385,10 @@ __global__ void __launch_bounds__(NT, MINB) march_kernel(const __grid_constant__
             if (!conv) atomicAdd(P.nonconv, 1);
         }
         scatter_wide(P, P.geos[S.pr.geo], S.pr, slot_f64(P, P.off_vcube), threadIdx.x, NT);
+        if (!conv) {  // an infinite or NaN al leaves NaN in the residual's quads off the ball, where zeros belong
+            float4* rq = hot_slot(P) + kMarchR * 2 * march_row(NT);
+            for (int k = threadIdx.x; k < (kMarchP - kMarchR) * 2 * march_row(NT); k += NT) rq[k] = f4zero();
+        }
         __syncthreads();
         if (P.phase_clk && threadIdx.x == 0) {
             const long long t3 = clock64();

@@ -42,3 +42,43 @@ def test_inner_solves_that_miss_their_target(torch, r, tol, opts):
     assert out["stats"]["n_nonconv"] == 0 and ref["stats"]["n_nonconv"] == 0
     np.testing.assert_allclose(out["pairs"]["e_pair"], ref["pairs"]["e_pair"], rtol=200 * tol, atol=1e-12)
     assert d_maxrel(out["D"], ref["D"]) <= 1e4 * tol
+
+
+# An inner target beyond FP32's range: squares underflow, 0 / 0 follows and some solves
+# end as NaN. Which ones depends on the pair alone, not on what its CTA solved before.
+@pytest.mark.parametrize("r,r_ns", [(12, 0), (16, 0), (24, 0), (28, 0), (20, 12)])
+def test_a_failed_solve_leaves_nothing_behind(torch, r, r_ns):
+    from paper_1911_10630_gb300.exx import Exx
+    w = _workload(r)
+    kw = dict(precision=1, preconditioner=1, inner_tol=1e-25)
+    if r_ns:
+        kw.update(radii_mode=2, r_pe_nonself=r_ns, r_me_nonself=r_ns + 4)
+    phi = torch.from_numpy(w.orbitals()).cuda()
+    cen, D = torch.from_numpy(np.ascontiguousarray(w.centers)).cuda(), torch.empty_like(phi)
+    ex = Exx(w.cell, w.grid, w.r_pair, w.r_pe, w.r_me, w.l_max, 1e-25, **kw)
+    ex.compute(phi, cen, D, allow_noconv=True)
+    first = ex.pairs()["e_pair"].copy()
+    assert np.isnan(first).any()
+    for _ in range(4):
+        ex.compute(phi, cen, D, allow_noconv=True)
+        np.testing.assert_array_equal(ex.pairs()["e_pair"], first)
+    ex.close()
+
+
+# one ball (several groups of columns, and one), two CTA sizes, a ball beside one of pair_kernel
+@pytest.mark.parametrize("r,r_ns", [(8, 0), (24, 0), (20, 12), (25, 12)])
+def test_a_context_recovers_from_nan_orbitals(torch, r, r_ns):
+    w = _workload(r, n=3, tol=1e-9)
+    phi = w.orbitals()
+    kw = dict(precision=1, preconditioner=1)
+    if r_ns:
+        kw.update(radii_mode=2, r_pe_nonself=r_ns, r_me_nonself=r_ns + 4)
+    ref = run_gpu(w, phi, torch=torch, **kw)
+    ex, good = ref["ex"], ref["dphi"]
+    cen, D = torch.from_numpy(np.ascontiguousarray(w.centers)).cuda(), torch.empty_like(good)
+    ex.compute(torch.full_like(good, float("nan")), cen, D, allow_noconv=True)
+    assert ex.stats()["n_nonfinite"] == ref["stats"]["n_pair"]
+    ex.compute(good, cen, D)
+    np.testing.assert_array_equal(ex.pairs()["e_pair"], ref["pairs"]["e_pair"])
+    assert d_maxrel(D.cpu().numpy(), ref["D"]) <= 1e-12  # the order of the atomic adds
+    ex.close()
