@@ -106,18 +106,15 @@ __device__ __forceinline__ double bound_of(unsigned top) {
     return top < 0x7ff00000u ? __hiloint2double((int)(top + 1u), 0) : __hiloint2double((int)top, 0);
 }
 
-// The fixed-point copy of v: v 2^k rounded, |v 2^k| <= 2^59, k >= 0. The scale is
-// added to v's exponent (a zero or denormal v stays below 1/2).
+// The fixed-point copy of v: v 2^k truncated, |v 2^k| <= 2^59 (k of either sign).
+// The scale is added to v's exponent (a zero or denormal v stays below 1/2; an
+// infinite or NaN v becomes 0: its pair ends on the sums of r and p).
 __device__ __forceinline__ long long to_fixed(double v, int k) {
-#if 1
     const int h = __double2hiint(v);
     const int e = (h >> 20) & 0x7ff;
     const unsigned long long m = ((unsigned long long)(unsigned)((h & 0xfffff) | 0x100000) << 32 | (unsigned)__double2loint(v)) << 7;
-    const long long t = (long long)(m >> min(1082 - k - e, 63));
+    const long long t = (long long)(m >> min((unsigned)(1082 - k - e), 63u));
     return h < 0 ? -t : t;
-#else
-    return __double2ll_rn(__hiloint2double(__double2hiint(v) + (k << 20), __double2loint(v)));
-#endif
 }
 
 // -180 delta^2 / 2^8 times lap p from the fixed-point copy, in units of the
@@ -336,7 +333,7 @@ __global__ void __launch_bounds__(NT, 1024 / NT) cg64_kernel(const __grid_consta
         const auto scale_for = [&](double bound) {  // |p| <= bound: |p 2^sh| <= 2^59
             int e = 0;
             (void)frexp(bound, &e);
-            sh = 59 - min(max(e, -900), 59);
+            sh = 59 - min(max(e, -900), 900);
             unit = ldexp(P.fix_inv, 8 - sh);
         };
         int it = 0;
