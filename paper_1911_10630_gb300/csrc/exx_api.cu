@@ -1176,7 +1176,7 @@ extern "C" exx_status exx_init(exx_ctx** out, const double cell[3], const int gr
         }
         for (int v = 0; v < cluster_variant_count(); ++v)
             if (need_smem[v] && (e = cluster_set_smem(v, need_smem[v])) != cudaSuccess)
-                return bail(cuda_fail(c, e, "cudaFuncSetAttribute(class shared memory)"));
+                return bail(cuda_fail(c, e, "shared-memory limit (radius classes)"));
         c->per_class = true;
         e = cudaMalloc(&c->d_class, sizeof(int) * 3 * (size_t)c->n_geo);
         if (e != cudaSuccess) return bail(cuda_fail(c, e, "cudaMalloc(radius classes)"));

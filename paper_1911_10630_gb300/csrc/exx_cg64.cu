@@ -412,7 +412,7 @@ size_t cg64_smem(int r_pe) { return sizeof(double) * 28 * (size_t)(2 * r_pe + 1)
 
 cudaError_t cg64_occupancy(int threads, bool fix, size_t smem, int* blocks_per_sm) {
     const void* f = cg64_fn(threads, fix);
-    cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = raise_smem_limit(f, smem);
     if (e != cudaSuccess) return e;
     return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, f, threads, smem);
 }

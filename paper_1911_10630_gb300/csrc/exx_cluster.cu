@@ -1843,7 +1843,7 @@ int cluster_variant(int C, int max_pts, int threads, int syz, bool iso) {
 
 cudaError_t cluster_prepare(int variant, size_t smem, int* max_clusters) {
     const ClusterVariant& K = kVariants[variant];
-    cudaError_t e = cudaFuncSetAttribute(K.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = raise_smem_limit(K.fn, smem);
     if (e != cudaSuccess) return e;
     if (K.c > 8) {  // clusters beyond the portable size of 8 need the opt-in
         e = cudaFuncSetAttribute(K.fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
@@ -1866,7 +1866,7 @@ cudaError_t cluster_prepare(int variant, size_t smem, int* max_clusters) {
 // Raises the variant's dynamic shared-memory limit (launch shapes of several
 // radius classes can share one variant).
 cudaError_t cluster_set_smem(int variant, size_t smem) {
-    return cudaFuncSetAttribute(kVariants[variant].fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    return raise_smem_limit(kVariants[variant].fn, smem);
 }
 
 cudaError_t launch_cluster_kernel(int variant, const SolveParams& P, const ClusterLayout& CL, int n_clusters,

@@ -4,8 +4,21 @@
 
 #include <cstdint>
 #include <cuda_runtime.h>
+#include <mutex>
 
 namespace exx {
+
+// Lets a kernel launch with so much dynamic shared memory. The limit belongs to the
+// function, which all contexts, networks and threads share: it is only ever raised,
+// as one that needs more may be alive. Occupancy and launches take their own size.
+inline cudaError_t raise_smem_limit(const void* kernel, size_t bytes) {
+    static std::mutex m;
+    std::lock_guard<std::mutex> lock(m);
+    cudaFuncAttributes at;
+    const cudaError_t e = cudaFuncGetAttributes(&at, kernel);
+    if (e != cudaSuccess || (size_t)at.maxDynamicSharedSizeBytes >= bytes) return e;
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+}
 
 // Multipole order limit and the Cartesian monomial count for l <= 6:
 // sum_{l=0..6} (l+1)(l+2)/2 = 84.

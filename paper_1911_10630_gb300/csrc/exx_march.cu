@@ -421,7 +421,7 @@ static const void* march_fn(int threads) {
 // shared memory, tensor memory and threads.
 cudaError_t march_occupancy(int threads, size_t smem, int* blocks_per_sm) {
     const void* f = march_fn(threads);
-    cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = raise_smem_limit(f, smem);
     if (e != cudaSuccess) return e;
     cudaFuncAttributes at;
     if ((e = cudaFuncGetAttributes(&at, f)) != cudaSuccess) return e;

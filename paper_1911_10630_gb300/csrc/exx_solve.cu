@@ -460,10 +460,9 @@ cudaError_t pair_kernel_occupancy(int threads, bool mixed, bool mg, bool one_bal
     else if (threads == 256) f = (const void*)pair_kernel<256, true>;
     else if (threads == 1024) f = (const void*)pair_kernel<1024, true>;
     else f = (const void*)pair_kernel<512, true>;
-    cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = raise_smem_limit(f, smem);
     if (e == cudaSuccess && mg && mixed && threads == 256)
-        e = cudaFuncSetAttribute((const void*)pair_kernel<512, true, true, false, true>,
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        e = raise_smem_limit((const void*)pair_kernel<512, true, true, false, true>, smem);
     if (e != cudaSuccess) return e;
     return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, f, threads, smem);
 }

@@ -955,7 +955,7 @@ static cudaError_t conv3_up(const __nv_bfloat16* x, const __nv_bfloat16* low, in
     a.n_stage = (int)std::min<size_t>(kStages, (room - fixed) / a.stage);
     if (a.n_stage < 1 || a.ncols > 512) return cudaErrorInvalidValue;
     const size_t smem = fixed + (size_t)a.n_stage * a.stage + 128;
-    UCK(cudaFuncSetAttribute(conv3_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    UCK(raise_smem_limit((const void*)conv3_tc_kernel, smem));
     conv3_tc_kernel<<<std::min(a.n_tiles, n_sm), kConvThreads, smem, st>>>(a);
     return cudaGetLastError();
 }
@@ -1131,7 +1131,7 @@ cudaError_t backward(Net& n, const float* in, const float* target, int B, cudaSt
         const int nsplit = dw_splits(B, s, kCin[l], kCout[l], n.n_sm);
         const int nb = dw_nb(kCout[l]), smem = 2 * dw_stage(nb);
         const auto f = nb == 16 ? dw_kernel<16> : dw_kernel<32>;
-        UCK(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+        UCK(raise_smem_limit((const void*)f, smem));
         dim3 grid(nsplit, kCin[l] / 16, kCout[l] / nb);
         const int count = 27 * kCin[l] * kCout[l] + kCout[l];
         f<<<grid, kDwThreads, smem, st>>>(x, low, cl, g, n.gpart, B, s, kCin[l], kCout[l], nsplit);
