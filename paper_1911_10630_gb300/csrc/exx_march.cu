@@ -181,7 +181,9 @@ __device__ __forceinline__ long long lap_int(const long long* __restrict__ f, in
 // FIX: lap v from the fixed-point copy (isotropic grids): the weights of Eq.
 // d2_1 times 180 delta^2 are the integers -490, 270, -27 and 2, so the sum is
 // exact, and three FP64 operations a point remain of 21. The copy rounds v at
-// 2^-51 to 2^-50 of its largest value.
+// 2^-51 to 2^-50 of its largest value, which bounds the residual at 1e-14 (R_PE 16) to
+// 1e-13 (R_PE 32) of the right-hand side; the FP64 stencil reaches 1e-14 throughout. A
+// pair whose residual does not halve goes on with the FP64 stencil.
 template <int NT, bool FIX>
 static __device__ __noinline__ double march_residual(const SolveParams& P, const PairState& S, float& rr) {
     const BallGeo& G = P.geos[S.pr.geo];
@@ -330,6 +332,16 @@ __global__ void __launch_bounds__(NT, MINB) march_kernel(const __grid_constant__
             __syncthreads();
             if (rn2 <= P.tol * P.tol * S.bb) break;
             const double rn = sqrt(rn2);
+            if (S.fix && S.refines > 0 && !(rn < 0.5 * S.rn_prev)) {
+                // the copy's rounding may bound this residual: the FP64 stencil from here on
+                __syncthreads();
+                if (threadIdx.x == 0) {
+                    S.fix = 0;
+                    S.rn_prev = 1e300;
+                }
+                __syncthreads();
+                continue;
+            }
             if (S.refines >= P.max_refine || S.iters >= P.max_iter || !(rn < S.rn_prev)) {
                 conv = false;
                 break;

@@ -44,6 +44,19 @@ def test_inner_solves_that_miss_their_target(torch, r, tol, opts):
     assert d_maxrel(out["D"], ref["D"]) <= 1e4 * tol
 
 
+# below what the fixed-point copy of v resolves: pairs go on with the FP64 stencil and
+# reach what it reaches
+@pytest.mark.parametrize("r,tol", [(16, 1e-14), (24, 3e-14), (24, 1e-14), (32, 1e-13), (32, 1e-14)])
+def test_the_integer_residual_reaches_what_the_fp64_one_reaches(torch, r, tol):
+    w = _workload(r, tol=tol)
+    phi = w.orbitals()
+    kw = dict(precision=1, preconditioner=1)
+    ref = run_gpu(w, phi, torch=torch, fixed_residual=1, **kw)
+    out = run_gpu(w, phi, torch=torch, **kw)
+    assert ref["stats"]["n_nonconv"] == 0 and out["stats"]["n_nonconv"] == 0
+    np.testing.assert_allclose(out["pairs"]["e_pair"], ref["pairs"]["e_pair"], rtol=200 * tol, atol=1e-15)
+
+
 # An inner target beyond FP32's range: squares underflow, 0 / 0 follows and some solves
 # end as NaN. Which ones depends on the pair alone, not on what its CTA solved before.
 @pytest.mark.parametrize("r,r_ns", [(12, 0), (16, 0), (24, 0), (28, 0), (20, 12)])
