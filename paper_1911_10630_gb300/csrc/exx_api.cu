@@ -134,8 +134,9 @@ struct exx_ctx {
     // the multigrid-preconditioned CG on clusters (preconditioner 1, precision 1):
     // mg_C CTAs per pair, mg_minb CTAs per SM, up to mg_clusters resident clusters
     int mg_C = 0, mg_minb = 2, mg_clusters = 0;
-    // the plain FP64 CG (exx_cg64.cu): CTAs that can be resident, 0 = not used
-    int cg64_ctas = 0;
+    // the plain FP64 CG (exx_cg64.cu): CTAs that can be resident, 0 = not used; CTAs
+    // per pair of the last call
+    int cg64_ctas = 0, cg64_team_last = 1;
     // the marching multigrid CG (exx_march.cu; preconditioner 1, precision 1,
     // solver_kind 0 or 1): one launch per CTA size, the largest balls first,
     // side by side on the context stream and the aux streams; each launch has
@@ -147,10 +148,11 @@ struct exx_ctx {
         SolveParams P;            // slot offsets and sizes of the class (the rest as in the context's P)
     };
     std::vector<MarchClass> march;
+    std::vector<int> march_rank;  // [n_geo] place of a ball in the order
     char* march_ws = nullptr;
     void* march_mem = nullptr;   // device tables
     int2* d_march_range = nullptr;
-    int* d_march_rank = nullptr; // [n_geo] place of a ball in the order (several classes)
+    int* d_march_rank = nullptr; // march_rank on the device
     bool march_general = false;  // one of the classes is pair_kernel's
     int pk_threads = 0;          // pair_kernel's threads
     int* d_march_cls = nullptr;  // [2 classes] start and length in the order, [classes] work counters
@@ -479,7 +481,7 @@ static cudaError_t launch_cg64(exx_ctx* c, const SolveParams& P, int n, cudaStre
     const int team = cg64_team(c, n);
     const int resident = std::max(1, c->cg64_ctas / team);
     const int teams = (int)std::min<long long>(std::min(c->n_slots, resident), (long long)n * (n + 1) / 2);
-    c->stats.cluster_size = team;
+    c->cg64_team_last = c->stats.cluster_size = team;
     c->stats.grid_ctas = teams * team;
     return launch_cg64_kernel(P, c->threads, cg64_fixed(c), teams, team, c->smem, st);
 }
@@ -608,6 +610,7 @@ static exx_status plan_march(exx_ctx* c, const std::vector<std::vector<HostMGLev
         c->march.push_back(K);
     }
     std::reverse(c->march.begin(), c->march.end());
+    c->march_rank = rank;
     std::vector<MarchGeo> mg;
     for (HostMarch& h : H) mg.push_back(h.G);
     std::memcpy(host.data(), mg.data(), sizeof(MarchGeo) * ng);
@@ -1393,6 +1396,22 @@ static exx_status ensure_pairs(exx_ctx* c, int n) {
 }
 
 // The launch sequence of one call (captured into a graph when batched).
+// P with a marching class's workspace.
+static SolveParams march_params(const exx_ctx* c, const exx_ctx::MarchClass& K, const SolveParams& P) {
+    SolveParams Pk = P;
+    Pk.ws = c->march_ws + K.at;
+    Pk.slot_bytes = K.P.slot_bytes;
+    Pk.ws_hot = c->march_ws + K.hot;
+    Pk.hot_bytes = K.P.hot_bytes;
+    Pk.off_vcube = K.P.off_vcube;
+    Pk.off_rho = K.P.off_rho;
+    Pk.off_vfix = K.P.off_vfix;
+    Pk.off_sy = K.P.off_sy;
+    Pk.off_ush = K.P.off_ush;
+    Pk.off_rows = K.P.off_rows;
+    return Pk;
+}
+
 static exx_status enqueue(exx_ctx* c, const double* orbitals, const double* centers, const double* alphas, int n,
                           double* d_xx, cudaStream_t st, bool capturing) {
     // inside a capture a plain event record only expresses a dependency; the
@@ -1489,16 +1508,7 @@ static exx_status enqueue(exx_ctx* c, const double* orbitals, const double* cent
                 CK(cudaStreamWaitEvent(st, c->march_ev[k - 1], 0), "cudaStreamWaitEvent(join)");
                 continue;
             }
-            Pk.ws = c->march_ws + K.at;
-            Pk.slot_bytes = K.P.slot_bytes;
-            Pk.ws_hot = c->march_ws + K.hot;
-            Pk.hot_bytes = K.P.hot_bytes;
-            Pk.off_vcube = K.P.off_vcube;
-            Pk.off_rho = K.P.off_rho;
-            Pk.off_vfix = K.P.off_vfix;
-            Pk.off_sy = K.P.off_sy;
-            Pk.off_ush = K.P.off_ush;
-            Pk.off_rows = K.P.off_rows;
+            Pk = march_params(c, K, Pk);
             CK(launch_march_kernel(Pk, K.threads, (int)std::min<long long>(K.slots, (long long)n * (n + 1) / 2), K.smem, ks),
                "marching pair kernel");
             if (k) {
@@ -2163,8 +2173,14 @@ extern "C" exx_status exx_debug_pair(exx_ctx* c, const double* orbitals, int ind
     P.refines = d_sc + 4;
     P.dbg_b = d_b;
     exx_status s = EXX_OK;
+    const exx_ctx::MarchClass* K = nullptr;  // the pair's marching class
+    for (const auto& k : c->march)
+        if (!k.general && c->march_rank[pr.geo] >= k.r_lo && c->march_rank[pr.geo] <= k.r_hi) K = &k;
+    if (K) P = march_params(c, *K, P);
+    // the kernel and the launch shape that solved the pair in the last call
     cudaError_t e = c->use_cluster ? launch_cluster_kernel(c->cl_variant, P, c->CL, 1, c->smem, st)
-                    : c->cg64_ctas ? launch_cg64(c, P, 1, st)
+                    : K            ? launch_march_kernel(P, K->threads, 1, K->smem, st)
+                    : c->cg64_ctas ? launch_cg64_kernel(P, c->threads, cg64_fixed(c), 1, c->cg64_team_last, c->smem, st)
                                    : launch_pair_kernel(P, c->pk_threads, c->opt.precision == 1, 1, c->smem, st);
     if (e == cudaSuccess) e = launch_debug_readback(P, pr, d_rho, d_v, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);

@@ -155,6 +155,7 @@ static __device__ __noinline__ double march_residual0(const SolveParams& P, cons
         const int k = __ldg(list + t);
         double r = kFourPi * rho[k];
         if (t < nrim) r += lap19<double>(vc, __ldg(cube + k), side, S2, st);
+        if (P.dbg_b) P.dbg_b[k] = r;
         const float f = (float)(r * scale);
         rq[__ldg(qidx + k)] = f;
         acc = fma(r, r, acc);
