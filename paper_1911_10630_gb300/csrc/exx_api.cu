@@ -1351,7 +1351,7 @@ extern "C" exx_status exx_init(exx_ctx** out, const double cell[3], const int gr
     P.inner_max_iter = o.inner_max_iter;
     P.inner_tol = o.inner_tol;
     P.max_refine = 40;
-    P.few = o.precision == 1 && o.preconditioner == 1 ? 2 * c->num_sms : 0;
+    P.few = o.precision == 1 && o.preconditioner == 1 && c->pk_threads == 256 && o.threads != 256 ? 2 * c->num_sms : 0;
     P.update_drop = o.update_drop;
     P.lmax = l_max;
     P.n_mono = (l_max + 1) * (l_max + 2) * (l_max + 3) / 6;
@@ -1913,6 +1913,7 @@ static exx_status finish_stats(exx_ctx* c, bool box) {
     CK(cudaMemcpy(sc, c->d_scalars, sizeof(sc), cudaMemcpyDeviceToHost), "read counters");
     const int npair = sc[0], nonconv = sc[2];
     c->stats.n_pair = npair;
+    if (c->march.empty() && c->P.few > 0 && !c->mg_C) c->stats.threads = npair <= c->P.few ? 512 : c->pk_threads;
     c->stats.n_nonconv = nonconv;
     c->stats.n_timeouts = sc[10];
     c->stats.n_nonfinite = sc[11];
