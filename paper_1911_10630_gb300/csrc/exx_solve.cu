@@ -352,7 +352,9 @@ __global__ void __launch_bounds__(NT, MG ? mg_min_blocks<NT, ONE_BALL, FEW>() : 
 
         // 6. E_ij over the PE ball and the D_xx scatter over the ME ball
         double e = 0.0;
-        for (int k = threadIdx.x; k < n_pe; k += NT) e = fma(rho[k], vc[cube[k]], e);
+        if constexpr (FEW) e = sum256(rho, vc, cube, n_pe);
+        else
+            for (int k = threadIdx.x; k < n_pe; k += NT) e = fma(rho[k], vc[cube[k]], e);
         e = block_sum<NT, double>(e, red, flip);
         if (threadIdx.x == 0) {
             P.e_pair[pidx] = e * P.dV;
