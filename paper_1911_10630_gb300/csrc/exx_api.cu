@@ -801,7 +801,7 @@ extern "C" exx_status exx_init(exx_ctx** out, const double cell[3], const int gr
     {
         std::vector<size_t> o_cube(c->n_geo), o_off(c->n_geo), o_rpe(c->n_geo), o_rme(c->n_geo), o_pl(c->n_geo),
             o_ro(c->n_geo), o_sn(c->n_geo), o_sf(c->n_geo), o_rim(c->n_geo), o_lay(c->n_geo), o_ir(c->n_geo),
-            o_bd(c->n_geo), o_bc(c->n_geo);
+            o_bd(c->n_geo), o_bc(c->n_geo), o_r2(c->n_geo);
         size_t at = 0;
         for (int g = 0; g < c->n_geo; ++g) {
             const HostBall& Bg = c->balls[g];
@@ -816,6 +816,7 @@ extern "C" exx_status exx_init(exx_ctx** out, const double cell[3], const int gr
             o_rim[g] = at; at = align256(at + sizeof(int) * Bg.rim.size());
             o_lay[g] = at; at = align256(at + sizeof(int) * Bg.layer.size());
             o_ir[g] = at; at = align256(at + sizeof(double) * Bg.layer_ir.size());
+            o_r2[g] = at; at = align256(at + sizeof(float) * Bg.row_r2.size());
             o_bd[g] = at; at = align256(at + sizeof(int) * Bg.duo.size());
             o_bc[g] = at; at = align256(at + sizeof(int) * Bg.duo_k.size());
         }
@@ -849,6 +850,7 @@ extern "C" exx_status exx_init(exx_ctx** out, const double cell[3], const int gr
             G.layer = (const int*)(gm + o_lay[g]);
             G.layer_ir = (const double*)(gm + o_ir[g]);
             G.n_layer = (int)Bg.layer.size();
+            G.row_r2 = (const float*)(gm + o_r2[g]);
             G.duo = (const int*)(gm + o_bd[g]);
             G.duo_k = (const int2*)(gm + o_bc[g]);
             G.n_duo = (int)Bg.duo.size();
@@ -860,6 +862,7 @@ extern "C" exx_status exx_init(exx_ctx** out, const double cell[3], const int gr
                 (e = cudaMemcpy(gm + o_pl[g], Bg.plane_pe.data(), sizeof(int) * Bg.plane_pe.size(), cudaMemcpyHostToDevice)) != cudaSuccess ||
                 (e = cudaMemcpy(gm + o_sn[g], Bg.sh_near.data(), sizeof(int) * Bg.sh_near.size(), cudaMemcpyHostToDevice)) != cudaSuccess ||
                 (e = cudaMemcpy(gm + o_sf[g], Bg.sh_far.data(), sizeof(int) * Bg.sh_far.size(), cudaMemcpyHostToDevice)) != cudaSuccess ||
+                (e = cudaMemcpy(gm + o_r2[g], Bg.row_r2.data(), sizeof(float) * Bg.row_r2.size(), cudaMemcpyHostToDevice)) != cudaSuccess ||
                 (e = cudaMemcpy(gm + o_rim[g], Bg.rim.data(), sizeof(int) * Bg.rim.size(), cudaMemcpyHostToDevice)) != cudaSuccess ||
                 (e = cudaMemcpy(gm + o_bd[g], Bg.duo.data(), sizeof(int) * Bg.duo.size(), cudaMemcpyHostToDevice)) != cudaSuccess ||
                 (e = cudaMemcpy(gm + o_bc[g], Bg.duo_k.data(), sizeof(int) * Bg.duo_k.size(), cudaMemcpyHostToDevice)) != cudaSuccess ||

@@ -178,8 +178,8 @@ void build_ball(HostBall& B, int r_pe, int r_me, int Rc) {
     B.n_me = (int)B.cube.size();
 }
 
-// The PE ball's rim first, the shell layer that its stencils read with 1 / r, and
-// (duos) the ball's points in pairs.
+// The PE ball's rim first, the shell layer that its stencils read with 1 / r, the ME
+// rows' x^2 + y^2, and (duos) the ball's points in pairs.
 void build_ball_layers(HostBall& B, int Rc, const double delta[3], bool duos) {
     B.rim.clear();
     const int in2 = B.r_pe > 3 ? (B.r_pe - 3) * (B.r_pe - 3) : -1;
@@ -206,8 +206,11 @@ void build_ball_layers(HostBall& B, int Rc, const double delta[3], bool duos) {
         }
     B.layer.clear();
     B.layer_ir.clear();
+    B.row_r2.clear();
     for (int row = 0; row < (int)B.rows_me.size(); ++row) {
         const RowRec& R = B.rows_me[row];
+        const double rx = R.ox * delta[0], ry = R.oy * delta[1];
+        B.row_r2.push_back((float)(rx * rx + ry * ry));
         for (int z = R.zpe + 1; z <= std::min<int>(R.zn, R.zme); ++z) {
             const double x = R.ox * delta[0], y = R.oy * delta[1], zz = z * delta[2];
             B.layer.push_back(row << 8 | z);

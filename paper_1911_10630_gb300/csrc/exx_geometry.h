@@ -21,6 +21,7 @@ struct HostBall {
     int n_rim = 0;
     std::vector<int> layer;         // shell points that the stencil reads: ME row << 8 | |z|
     std::vector<double> layer_ir;   // and their 1 / r
+    std::vector<float> row_r2;      // x^2 + y^2 of the ME rows
     std::vector<int> duo, duo_k;    // PE points in pairs along z, by bands of kBand rows in y
 };
 

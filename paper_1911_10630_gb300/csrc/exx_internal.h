@@ -66,6 +66,7 @@ struct BallGeo {
     const int* layer;
     const double* layer_ir;
     int n_layer;
+    const float* row_r2;     // [n_rows_me] x^2 + y^2, rounded once
     // The PE points in pairs (z even and odd), by bands of kBand rows in y, then
     // x, y, z: [n_duo] index of the first in a cube with rows of S + 1 (times 4;
     // bits 0, 1: the points on the ball), [n_duo] the two's compact indices (-1: none)

@@ -463,7 +463,8 @@ static __device__ __noinline__ void moment_rows_folded(const SolveParams& P, con
 // FP64, z and -z together: the even and odd parts of the P_l share the powers
 // of 1 / r^2, and 1 / r of every layer point comes from a table of the ball (33
 // FP64 operations for two points; 86 one by one with the root). The rest of
-// the shell only feeds D_xx: FP32, from the FP32 copy of U. Returns this
+// the shell only feeds D_xx: FP32, from the FP32 copies of U and of the row's FP64 x^2
+// + y^2. Returns this
 // thread's largest |v| on the layer.
 static __device__ __noinline__ void shell_planes(const SolveParams& P, const BallGeo& G, const double* __restrict__ T,
                                                  double* __restrict__ V, int tid, int nthr) {
@@ -502,7 +503,7 @@ static __device__ __noinline__ double shell_values(const SolveParams& P, const B
                                                    int nthr) {
     const int nr = G.n_rows_me, Rc = P.Rc;
     const RowRec* __restrict__ rows = G.rows_me;
-    const double dx = P.delta[0], dy = P.delta[1], dz = P.delta[2];
+    const double dz = P.delta[2];
     const long long S2 = P.S2, side = P.S;
     double big = 0.0;
     for (int q = tid; q < G.n_layer; q += nthr) {
@@ -540,8 +541,8 @@ static __device__ __noinline__ double shell_values(const SolveParams& P, const B
         const int pk = __ldg(G.sh_far + q), row = pk >> 8, z = (pk & 255) - 128;
         const RowRec R = rows[row];
         const float* __restrict__ U = U32 + row;
-        const float x = R.ox * (float)dx, y = R.oy * (float)dy, zz = (float)z * (float)dz;
-        const float ir = rsqrtf(fmaf(zz, zz, fmaf(x, x, y * y))), ir2 = ir * ir;
+        const float zz = (float)z * (float)dz;
+        const float ir = rsqrtf(fmaf(zz, zz, __ldg(G.row_r2 + row))), ir2 = ir * ir;
         float acc = 0.0f;
 #pragma unroll
         for (int l = kLmaxMax; l >= 0; --l) {
