@@ -63,6 +63,9 @@ struct ConvArgs {
 // SM 1.2; like this 0.85.
 constexpr int kEpilogue = 256, kProducers = 256, kConvThreads = kEpilogue + 32 + kProducers;
 
+// Index: of a voxel within a sample, long long for samples beyond 2^31 elements (in the
+// staging warps, whose address arithmetic then costs 2 % of the forward pass).
+template <typename Index>
 __global__ void __launch_bounds__(kConvThreads, 1) conv3_tc_kernel(const __grid_constant__ ConvArgs a) {
     extern __shared__ unsigned char smem_dyn[];
     __shared__ uint64_t full[kStages], empty[kStages], acc_full[2], acc_empty[2], wres;
@@ -164,7 +167,7 @@ __global__ void __launch_bounds__(kConvThreads, 1) conv3_tc_kernel(const __grid_
                     const bool in =
                         (unsigned)d < (unsigned)a.D && (unsigned)h < (unsigned)a.H && (unsigned)w < (unsigned)a.W;
                     const __nv_bfloat16* src =
-                        in ? xb + (size_t)(((d >> sh) * H + (h >> sh)) * W + (w >> sh)) * ch + o * 8 : a.x;
+                        in ? xb + (size_t)(((Index)(d >> sh) * H + (h >> sh)) * W + (w >> sh)) * ch + o * 8 : a.x;
                     tc::cp_async16(st + (size_t)o * a.itile + (size_t)(row * kWW + wx) * 16, src, in ? 16u : 0u);
                 }
                 tc::cp_async_commit();
@@ -942,7 +945,7 @@ static cudaError_t conv3_up(const __nv_bfloat16* x, const __nv_bfloat16* low, in
             tiles = n;
         }
     }
-    if (tiles > 0x7fffffffLL || (long long)D * H * W * cin > 0x7fffffffLL) return cudaErrorInvalidValue;
+    if (tiles > 0x7fffffffLL) return cudaErrorInvalidValue;
     a.n_tiles = (int)tiles;
     a.tiles_d = (D + a.DT - 1) / a.DT;
     a.acc_cols = (a.DT + (a.fold ? 4 : 0)) * a.nb;
@@ -955,8 +958,9 @@ static cudaError_t conv3_up(const __nv_bfloat16* x, const __nv_bfloat16* low, in
     a.n_stage = (int)std::min<size_t>(kStages, (room - fixed) / a.stage);
     if (a.n_stage < 1 || a.ncols > 512) return cudaErrorInvalidValue;
     const size_t smem = fixed + (size_t)a.n_stage * a.stage + 128;
-    UCK(raise_smem_limit((const void*)conv3_tc_kernel, smem));
-    conv3_tc_kernel<<<std::min(a.n_tiles, n_sm), kConvThreads, smem, st>>>(a);
+    const auto kernel = (long long)D * H * W * cin > 0x7fffffffLL ? conv3_tc_kernel<long long> : conv3_tc_kernel<int>;
+    UCK(raise_smem_limit((const void*)kernel, smem));
+    kernel<<<std::min(a.n_tiles, n_sm), kConvThreads, smem, st>>>(a);
     return cudaGetLastError();
 }
 
