@@ -101,8 +101,9 @@ typedef struct {
                           or 1024 (other values: the library choice, 512, or
                           for the FP32 multigrid CG 128, 256 or 512 by the
                           size of the pair's ball, 256 or 512 for the largest
-                          of the context), the cluster solver only the launch
-                          shapes it is built for.                             */
+                          of the context; 1024: the general kernel only), the
+                          cluster solver only the launch shapes it is built
+                          for.                                                */
     int ctas_per_sm;   /* resident CTAs per SM, 0 = library choice (the
                           multigrid CG on clusters: 1 or 2, default 2).         */
     int solver_kind;   /* 0 = library choice; 1 = one CTA per pair with state in

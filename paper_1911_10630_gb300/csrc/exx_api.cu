@@ -501,14 +501,23 @@ static bool march_steady(int R) {
     return over <= 1;
 }
 
+// The smallest ball that gains from marching, by the threads a CTA (0: the library's
+// choice): below it the planes are a few columns each and their barriers are the
+// time. Milliseconds marching / on pair_kernel for 36 and 820 pairs: R_PE 4 0.54 / 0.31
+// and 1.48 / 0.90, 6 0.67 / 0.50 and 2.0 / 1.6, 7 0.76 / 0.59 and 2.4 / 2.1, 8 0.72 /
+// 0.70 and 2.38 / 2.48. With 512 threads asked for, 36 and 465 pairs: R_PE 12 1.37 / 1.76
+// and 5.2 / 4.8, 14 1.6 / 2.6 and 6.3 / 7.3.
+static int march_from(int threads) { return threads == 512 ? 14 : 8; }
+
 // Plans the marching multigrid CG: classes of radii by CTA size, tables and
 // slot layouts. Leaves c->march empty when a ball has no coarse level or is
 // larger than the largest CTA holds, when the requested threads do not hold
-// the largest ball's columns, or when no ball is steady (pair_kernel then runs
-// the call).
+// the largest ball's columns or are 1024 (one CTA of 64 registers a thread: R_PE 16
+// 9.1 ms, pair_kernel 5.4), or when no ball gains (pair_kernel then runs the call).
 static exx_status plan_march(exx_ctx* c, const std::vector<std::vector<HostMGLevel>>& mgl) {
     const int ng = c->n_geo, want = c->opt.threads;
-    const bool asked = want == 256 || want == 512 || want == 1024;
+    const bool asked = want == 256 || want == 512;
+    if (want == 1024) return EXX_OK;
     std::vector<HostMarch> H(ng);
     std::vector<int> nt(ng, 0);  // 0: pair_kernel
     const int largest = march_threads(march_columns(c->balls[ng - 1].r_pe));
@@ -516,7 +525,7 @@ static exx_status plan_march(exx_ctx* c, const std::vector<std::vector<HostMGLev
     for (int g = 0; g < ng; ++g) {
         const int R = c->balls[g].r_pe;
         if (R > 35 || R <= 3) return EXX_OK;
-        if (!march_steady(R)) {
+        if (R < march_from(asked ? want : 0) || !march_steady(R)) {
             c->march_general = true;
             H[g].G = MarchGeo();
             continue;
@@ -1354,7 +1363,10 @@ extern "C" exx_status exx_init(exx_ctx** out, const double cell[3], const int gr
     P.inner_max_iter = o.inner_max_iter;
     P.inner_tol = o.inner_tol;
     P.max_refine = 40;
-    P.few = o.precision == 1 && o.preconditioner == 1 && c->pk_threads == 256 && o.threads != 256 ? 2 * c->num_sms : 0;
+    // few pairs on 512 threads (exx_solve.cu): the library's choice only, and not for contexts of balls below
+    // R_PE 8, a few points a thread, whose calls keep the default of 256 (0.61 against 0.50 ms at R_PE 6)
+    const bool choose = o.precision == 1 && o.preconditioner == 1 && c->pk_threads == 256 && o.threads != 256;
+    P.few = choose && r_pe >= 8 ? 2 * c->num_sms : 0;
     P.update_drop = o.update_drop;
     P.lmax = l_max;
     P.n_mono = (l_max + 1) * (l_max + 2) * (l_max + 3) / 6;

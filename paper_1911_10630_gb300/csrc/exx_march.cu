@@ -424,8 +424,7 @@ static const void* march_fn(int threads) {
     switch (threads) {
         case 128: return (const void*)march_kernel<128, 4>;
         case 256: return (const void*)march_kernel<256, 2>;
-        case 512: return (const void*)march_kernel<512, 1>;
-        default: return (const void*)march_kernel<1024, 1>;
+        default: return (const void*)march_kernel<512, 1>;
     }
 }
 
@@ -445,8 +444,7 @@ cudaError_t march_occupancy(int threads, size_t smem, int* blocks_per_sm) {
         (e = cudaDeviceGetAttribute(&most, cudaDevAttrMaxThreadsPerMultiProcessor, dev)) != cudaSuccess)
         return e;
     const int warp_regs = (at.numRegs * 32 + 255) & ~255;
-    const int tm = threads == 128 ? ring_columns<128>() : threads == 256 ? ring_columns<256>()
-                   : threads == 512 ? ring_columns<512>() : ring_columns<1024>();
+    const int tm = threads == 128 ? ring_columns<128>() : threads == 256 ? ring_columns<256>() : ring_columns<512>();
     const int cta = (int)((smem + at.sharedSizeBytes + 1024 + 127) & ~(size_t)127);
     *blocks_per_sm = std::min(std::min(regs / (warp_regs * (threads / 32)), bytes / cta), std::min(most / threads, 512 / tm));
     return cudaSuccess;

@@ -1,5 +1,5 @@
-"""Which kernel takes a ball: the FP32 multigrid CG marches balls from R_PE 4 to 32 whose
-hierarchy is steady, in CTAs of 128, 256 or 512 threads (four, two, one per SM; the
+"""Which kernel takes a ball: the FP32 multigrid CG marches balls from R_PE 8 to 32 whose
+hierarchy is steady (from 14 with 512 threads asked for, none with 1024), in CTAs of 128, 256 or 512 threads (four, two, one per SM; the
 largest ball's class at least 256), and leaves the others to the general kernel (six CTAs
 per SM with one ball, five with several). grid_ctas and threads tell them apart. Then
 calls of all classes at once in which every slot takes several pairs of different balls,
@@ -34,14 +34,16 @@ def _init(r, **kw):
 @pytest.mark.parametrize("r", range(1, 38))
 def test_the_kernel_of_a_ball(torch, r):
     sms = torch.cuda.get_device_properties(0).multi_processor_count
-    if r <= 3 or r > 32 or r in GENERAL:
+    if r < 8 or r > 32 or r in GENERAL:
         assert _init(r) == (256, 6 * sms)
     elif r <= 24:
         assert _init(r) == (256, 2 * sms)
     else:
         assert _init(r) == (512, sms)
-    if r > 3 and r <= 16 and r not in GENERAL:  # CTA sizes asked for
-        assert _init(r, threads=512) == (512, sms) and _init(r, ctas_per_sm=1) == (256, sms)
+    if 8 <= r <= 16 and r not in GENERAL:  # CTA sizes asked for
+        assert _init(r, threads=512) == ((512, sms) if r >= 14 else (512, 2 * sms))
+        assert _init(r, threads=1024) == (1024, sms)
+        assert _init(r, ctas_per_sm=1) == (256, sms)
 
 
 @pytest.mark.parametrize("per_sm", [0, 1])
