@@ -802,8 +802,10 @@ extern "C" exx_status exx_init(exx_ctx** out, const double cell[3], const int gr
             Rm = g == 0 ? o.r_me_nonself : r_me;
         }
         build_ball(c->balls[g], R, Rm, Rc);
-        // what the plain FP64 CG and the marching kernel read
-        if (o.precision == 0 || o.preconditioner == 1) build_ball_layers(c->balls[g], Rc, c->delta, o.precision == 0);
+        // what the plain FP64 CG (duos) and the marching kernel (rim) read
+        if (o.precision == 0 && o.preconditioner == 0) build_ball_layers(c->balls[g], Rc, c->delta, false, true);
+        else if (o.precision == 1 && o.preconditioner == 1 && o.solver_kind != 2)
+            build_ball_layers(c->balls[g], Rc, c->delta, true, false);
     }
     c->hb = c->balls.back();
     const HostBall& B = c->hb;

@@ -178,12 +178,12 @@ void build_ball(HostBall& B, int r_pe, int r_me, int Rc) {
     B.n_me = (int)B.cube.size();
 }
 
-// The PE ball's rim first, the shell layer that its stencils read with 1 / r, the ME
-// rows' x^2 + y^2, and (duos) the ball's points in pairs.
-void build_ball_layers(HostBall& B, int Rc, const double delta[3], bool duos) {
+// The shell layer that the PE ball's stencils read with 1 / r, the ME rows' x^2 + y^2,
+// and (rim) the ball's points with its rim first, (duos) its points in pairs.
+void build_ball_layers(HostBall& B, int Rc, const double delta[3], bool rim, bool duos) {
     B.rim.clear();
     const int in2 = B.r_pe > 3 ? (B.r_pe - 3) * (B.r_pe - 3) : -1;
-    for (int pass = 0; pass < 2; ++pass) {
+    for (int pass = 0; rim && pass < 2; ++pass) {
         for (int k = 0; k < B.n_pe; ++k) {
             const int x = (B.off[k] & 255) - 128, y = ((B.off[k] >> 8) & 255) - 128, z = ((B.off[k] >> 16) & 255) - 128;
             if ((x * x + y * y + z * z > in2) == (pass == 0)) B.rim.push_back(k);

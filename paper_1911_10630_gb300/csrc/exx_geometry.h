@@ -36,7 +36,7 @@ void build_multipole_const(MultipoleConst& mc);
 bool build_cluster_layout(const HostBall& B, int C, ClusterLayout& L, std::vector<int>& pt_slab, bool pitch4 = false,
                           int max_planes = 0);
 void build_ball(HostBall& B, int r_pe, int r_me, int Rc);
-void build_ball_layers(HostBall& B, int Rc, const double delta[3], bool duos);
+void build_ball_layers(HostBall& B, int Rc, const double delta[3], bool rim, bool duos);
 
 // Thread-slot maps of the cluster solver for NT threads x PTS points per CTA:
 // slot (j, t) of CTA r holds one point of the CTA's slab. Points are dealt so
