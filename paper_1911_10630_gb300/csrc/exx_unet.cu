@@ -921,6 +921,10 @@ static cudaError_t conv3_up(const __nv_bfloat16* x, const __nv_bfloat16* low, in
     // and the deepest level has tiles for all SMs.
     a.nsplit = 1;
     while (cout / a.nsplit > 64 || cout % (16 * a.nsplit)) ++a.nsplit;
+    // 80, 112, 176 and 208 have no even split but slices of 16, each of which would stage
+    // the input again: one slice and one stage (exx_unet_conv3d, 112 to 112 channels on
+    // 3 x 200 x 200: 0.26 ms, 0.51 in slices).
+    if (cout / a.nsplit < 32 && cout > 64) a.nsplit = 1;
     a.nb = cout / a.nsplit;
     a.wtile = 27u * (uint32_t)a.nb * 32u;
     a.tiles_w = (W + kTW - 1) / kTW;
@@ -934,7 +938,7 @@ static cudaError_t conv3_up(const __nv_bfloat16* x, const __nv_bfloat16* low, in
     const int most = a.fold ? (cout <= 16 ? 8 : 4) : 4;
     double best = 0.0;
     long long tiles = 0;
-    for (int DT = 1; DT <= most && DT <= D; ++DT) {
+    for (int DT = 1; DT <= most && DT <= D && (a.fold || DT * a.nb <= 512); ++DT) {
         const long long n = (long long)a.tiles_w * a.tiles_h * ((D + DT - 1) / DT) * B * a.nsplit;
         const double mma = (a.fold ? 9.0 * (DT + 2) : 27.0 * DT) * std::max(40.0, 0.55 * a.nb * (a.fold ? 3 : 1));
         const double load = 110.0 * (DT + 2) + (a.resident ? 0.0 : a.wtile / 64.0);
