@@ -111,11 +111,12 @@ struct MGGeo {
 // Level 1 marches from radius 6 on, the levels below it from 9: smaller ones
 // live in shared memory as cubes.
 constexpr int kMarchSmem1 = 5, kMarchSmem = 8;
-constexpr int kMarchMax = 3;    // marching levels at most (R_PE <= 35: 35, 18, 9)
+constexpr int kMarchMax = 2;    // marching levels at most (the largest ball that marches, R_PE 32: 32, 16)
 // A vector in the hot slot: two rows of march_row quads, a constant of the CTA
-// size (the quads of the largest ball that its threads hold), so that the
-// vectors' places are constants of the kernel; level 0's vectors in this order.
-constexpr int march_row(int threads) { return threads <= 128 ? 2816 : threads <= 256 ? 8704 : 23552; }
+// size (the quads of the largest ball that marches on its threads: R_PE 16, 24, 32),
+// so that the vectors' places are constants of the kernel; level 0's vectors in this
+// order.
+constexpr int march_row(int threads) { return threads <= 128 ? 2816 : threads <= 256 ? 8704 : 19456; }
 enum { kMarchR = 0, kMarchP = 2, kMarchZ = 4, kMarchD = 5, kMarchAp = 6, kMarchVectors = 7 };  // R, P: two each
 constexpr int kMarchPts = 9;    // points per thread of a shared-memory level at most
 struct MarchLv {
