@@ -514,9 +514,10 @@ exx_status exx_mg_levels(int r_pe, const double delta[3], int *radius, int *poin
                          double *minv, size_t minv_cap);
 
 /*
- * Measures the FP64 FMA rate of the current device, the roofline denominator
- * of the plain FP64 CG (whose binding unit on this GPU is the FP64 pipe, not
- * HBM). The paper has no counterpart. Eight independent FMA chains per thread
+ * Measures the FP64 FMA rate of the current device: the roofline denominator of
+ * the FP64 stencil (the plain FP64 CG on anisotropic grids; on isotropic ones its
+ * integer stencil leaves DRAM and latency as the bound), and of the equivalent FP64
+ * rate that is quoted beside it. The paper has no counterpart. Eight independent FMA chains per thread
  * on 8 CTAs of 256 threads per SM; the best of three timed launches.
  *   tflops   host, receives 2 x FMAs / s / 1e12
  *   stream   cudaStream_t, NULL = legacy default stream; the call waits for it

@@ -489,12 +489,15 @@ static cudaError_t launch_cg64(exx_ctx* c, const SolveParams& P, int n, cudaStre
 // CTA size of the marching multigrid CG for a ball of n columns: one each.
 static int march_threads(int n) { return n <= 128 ? 128 : (n <= 256 ? 256 : 512); }
 
-// Whether a ball's multigrid PCG holds in FP32: at most one of its coarse balls
-// reaches beyond its fine one (2 R_{l+1} > R_l). Where two do, the PCG carries
-// rounding errors of 1e-7 up a hundredfold, so that every order of its sums stops
-// somewhere else within the tolerance: at tol 1e-8, D_xx on another CTA size differs
-// by 7e-10 to 1.2e-9 (R_PE 17, 21, 25, 34), against 1e-11 (16, 24, 32). Those balls
-// stay on pair_kernel, whose results callers have.
+// Whether a ball's FP32 multigrid PCG gives the same result in every order of its
+// sums: at most one of its coarse balls reaches beyond its fine one (2 R_{l+1} > R_l).
+// Where two do, the PCG carries rounding errors of 1e-7 up a hundredfold, and every
+// order of the sums stops somewhere else within the tolerance: at tol 1e-8, D_xx on
+// another CTA size of the same kernel differs by 7e-10 to 1.2e-9 (R_PE 17, 21, 25,
+// 34), against 1e-11 (16, 24, 32). The error against the exact solution is the same
+// either way. Such balls stay on pair_kernel so that results hold still to 1e-9, not
+// for accuracy; they cost a factor of 1.5 to 3 in time (269 pairs at R_PE 19 and 25:
+// 27 ms, marching 9).
 static bool march_steady(int R) {
     int over = 0;
     for (; R > 3; R = (R + 1) / 2) over += R & 1;

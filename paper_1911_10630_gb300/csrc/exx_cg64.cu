@@ -6,24 +6,26 @@
 // 24 operations per point and iteration, 19 of them the stencil. On isotropic
 // grids A p is formed in integers instead: the weights of Eq. d2_1 times
 // 180 delta^2 are -490, 270, -27 and 2, and p is kept a second time as a 60-bit
-// fixed-point number under a bound that the CG's own reductions give each
-// iteration. The sum is exact but for its last 8 of 71 bits, and one conversion
-// turns it back: 7 FP64 operations a point in all. The error of A p is 2^-51 of
-// the largest |p| over 180 delta^2; the FP64 stencil's is a few 2^-53 of each of
-// 19 terms of up to 1470 / 180 |p| / delta^2.
+// fixed-point number under a bound B that the CG's own reductions give each
+// iteration (a power of 2, up to 4 times the largest |p|). The sum is exact but for
+// its last 8 of 71 bits, and one conversion turns it back: 7 FP64 operations a point
+// in all. The copy is truncated at 2^-59 B, so A p is off by (3264 + 256) 2^-59 B over
+// 180 delta^2 at most, 2^-47 B: values below 2^-6 B have fewer bits in it than in FP64.
+// Over the directions of CGs on balls of R_PE 8, 16 and 24 the error of A p (2-norm)
+// is 4e-17 to 5e-16 of it; the FP64 stencil's, whose rounded weights do not sum to
+// zero, 2e-16 to 6e-15.
 //
 // Two points along z share their loads (17 of 16 bytes instead of 38 of 8). What
-// is left is bound by latency and DRAM: 116 bytes a point and iteration, two
+// is left is bound by latency and DRAM: 100 bytes a point and iteration, two
 // thirds of the copy rate, and A p's loads. Several CTAs on a pair keep all SMs
 // busy on few pairs.
 //
 // Milliseconds, 64 orbitals at R_PE 24 (755 pairs, 158 iterations) / 8 orbitals
 // at R_PE 16 (36 pairs, 134): cg_ball 358 / 20.1; integers one point at a time,
 // 10 FP64 operations 186 / 4.2 (teams of 2 / 4); 7 operations 176 / 3.9; in
-// pairs 164 / 3.5. Of 168, A p takes 81, the residual 33, the direction 37 and
-// the team's barriers 17.
+// pairs 165 / 3.4; the sums' additions on one warp 155 / 3.2. Of 165, A p took 81, the
+// residual 33, the direction 37 and the team's barriers 17.
 #include <cuda_runtime.h>
-
 
 #include "exx_phases.cuh"
 
@@ -134,7 +136,7 @@ __device__ __forceinline__ long long to_fixed(double v, int k) {
 // -180 delta^2 / 2^8 times lap p from the fixed-point copy, in units of the
 // copy: m the value, s1 to s3 the sums of its neighbours at distance 1 to 3
 // (they fit 64 bits). The weighted sum (71 bits) is formed in two limbs and
-// loses its last 8 bits: 2^-51 of the largest |p| over 180 delta^2.
+// loses its last 8 bits.
 __device__ __forceinline__ double weigh_fixed(long long m, long long s1, long long s2, long long s3) {
     const auto lo = [](long long v) { return (long long)(unsigned)v; };
     const auto hi = [](long long v) { return (long long)(int)(v >> 32); };

@@ -8,14 +8,16 @@
 // up-sampling and concatenation with the skip tensor up, a 1x1x1 head.
 // Activations and weights are BF16 in channels-last layout, accumulation FP32.
 //
-// The 3x3x3 convolutions (all but the 2-channel input layer) are implicit GEMMs
-// on the tcgen05 tensor cores: one CTA computes a 16 (H) x 8 (W) x DT (D)
-// output tile for all output channels, the input halo tile and the weights of
-// one 16-channel chunk are staged in shared memory as 8-row core matrices, and
-// each of the 27 taps is one MMA (M = 128 voxels, N = cout, K = 16) whose A
-// operand is the same staged tile seen through a shifted descriptor. The
-// accumulators live in tensor memory and are read back with tcgen05.ld for
-// the bias / ReLU / mask epilogue.
+// The 3x3x3 convolutions (all but the 3-channel input layer) are implicit GEMMs
+// on the tcgen05 tensor cores: persistent CTAs, one per SM, compute 16 (H) x 8 (W)
+// x DT (D) output tiles of a slice of the output channels. The input halo tile and
+// the weights of one 16-channel chunk are staged in shared memory as 8-row core
+// matrices, and each of the 27 taps is one MMA (M = 128 voxels, N = the slice,
+// K = 16; three depth taps in one for up to 32 channels) whose A operand is the same
+// staged tile seen through a shifted descriptor. The up-path layers read the
+// up-sampled and the skip tensor in place of a concatenated one. The accumulators
+// live in tensor memory and are read back with tcgen05.ld for the bias / ReLU / mask
+// epilogue.
 #include "exx_unet.cuh"
 #include "exx_unet_tc.cuh"
 #include "exx_phases.cuh"  // the multipole constants (this unit's copy of c_mp)
@@ -522,8 +524,8 @@ __global__ void __launch_bounds__(32 * K) reduce_parts_kernel(const float* __res
     }
 }
 cudaError_t reduce_parts(const float* part, int n_parts, long long stride, int count, float* out, cudaStream_t st) {
-    // 32 threads an output only for long chains: 19 parts of 442,000 outputs take 56
-    // us with 32 threads, 20 with 4
+    // 32 threads an output only for long chains (19 parts of 442,000 outputs: 56 us with
+    // 32 threads, 20 with 4); 8 up to 128 parts
     if (n_parts > 128) reduce_parts_kernel<32><<<(count + 31) / 32, dim3(32, 32), 0, st>>>(part, n_parts, stride, count, out);
     else reduce_parts_kernel<8><<<(count + 31) / 32, dim3(32, 8), 0, st>>>(part, n_parts, stride, count, out);
     return cudaGetLastError();
@@ -884,7 +886,7 @@ size_t param_count() { return param_offset(kLayers); }
 
 // Whether a convolution with n_out output channels folds its depth taps (one
 // MMA of N = 3 n_out per (dh, dw)): N <= 256 and the depth-shifted TMEM slices
-// of a tile within 256 columns (two CTAs per SM).
+// of a tile within 256 columns, so that two accumulators fit.
 static bool conv_folds(int n_out) { return n_out <= 32; }
 
 cudaError_t pack_weights(const float* w, __nv_bfloat16* wp, int cin, int cout, int flip, cudaStream_t st) {
