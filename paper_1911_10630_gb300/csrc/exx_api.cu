@@ -805,8 +805,8 @@ extern "C" exx_status exx_init(exx_ctx** out, const double cell[3], const int gr
             Rm = g == 0 ? o.r_me_nonself : r_me;
         }
         build_ball(c->balls[g], R, Rm, Rc);
-        // what the plain FP64 CG (duos) and the marching kernel (rim) read
-        if (o.precision == 0 && o.preconditioner == 0) build_ball_layers(c->balls[g], Rc, c->delta, false, true);
+        // what the plain FP64 CG (duos; also where no ball has a coarse level) and the marching kernel (rim) read
+        if (o.precision == 0 && (o.preconditioner == 0 || r_pe <= 3)) build_ball_layers(c->balls[g], Rc, c->delta, false, true);
         else if (o.precision == 1 && o.preconditioner == 1 && o.solver_kind != 2)
             build_ball_layers(c->balls[g], Rc, c->delta, true, false);
     }
