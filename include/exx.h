@@ -152,7 +152,9 @@ typedef struct {
                           iteration, do not overflow), on an isotropic
                           grid: 0 = the FP64 residuals of the refinement come
                           from an exact integer stencil on a fixed-point copy
-                          of v (default), 1 = from the FP64 stencil, 2 = test
+                          of v (default; the FP32 multigrid CG goes on with the
+                          FP64 stencil where the copy's rounding stalls a pair),
+                          1 = from the FP64 stencil, 2 = test
                           mode: the fixed-point bound is made too small, so
                           every pair takes the overflow fallback to the FP64
                           stencil.                                              */
@@ -204,7 +206,7 @@ typedef struct {
     int solver_kind;       /* solver that ran                                      */
     int cluster_size;      /* CTAs per pair                                        */
     int grid_ctas;         /* CTAs launched for the pair kernel                    */
-    int threads;           /* threads per CTA                                      */
+    int threads;           /* threads per CTA (several sizes: the largest ball's)  */
     double phase_ms[4];    /* the pair-kernel time split by the cycle counts of
                               its CTAs (clusters) into setup (gather,
                               multipoles, shell), the FP64 residuals of the
@@ -356,8 +358,9 @@ exx_status exx_get_pairs(const exx_ctx *ctx, int *pi, int *pj, int *g, int *radi
  *   b         host [N_PE]: right-hand side 4 pi rho + boundary charge of
  *             Eq. pe_mat_red written as A v = b (may be NULL)
  * Ball points are in Algorithm 2 order (lexicographic (x, y, z) within the PE
- * ball, then within the shell). Re-solves the pair on the device with the
- * context's options. EXX_ENOPAIR if index is out of range.
+ * ball, then within the shell). Re-solves the pair on the device with the kernel
+ * and launch shape of the last call, whose stats stay. EXX_ENOPAIR if index is
+ * out of range.
  */
 exx_status exx_debug_pair(exx_ctx *ctx, const double *orbitals, int index, double *rho, double *v,
                           double *b, void *stream);

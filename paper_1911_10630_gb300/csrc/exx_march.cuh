@@ -31,8 +31,8 @@
 // in pairs; the next planes are staged by cp.async.
 //
 // What bounds it: latency. A plane is one step, with a barrier, of every thread of the
-// pair; counters give 24 % of the DRAM rate, 1.5 instructions a clock, and the waits
-// on staged planes and on the barrier as the first stalls. 128 registers a thread
+// pair; over the kernel the counters give 24 % of the DRAM rate, 0.8 instructions a
+// clock and SM, and the waits on staged planes and on the barrier as the first stalls. 128 registers a thread
 // leave 16 warps to an SM to cover them. Per pair and iteration
 // at R_PE 24, microseconds of an SM: 340 for the sweeps kept apart (the
 // pair_kernel form); 225 with one row per column; 190 with the ring in
